@@ -347,7 +347,10 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *   6  FP64 arithmetic throughput of the GPU: TFLOP/s of DFMA on the CUDA
  *      cores and of mma.sync m8n8k4 f64 (each the best of three launches of
  *      8 blocks of 256 threads per SM, 2 flops per FMA), the SM count and
- *      the number of blocks */
+ *      the number of blocks
+ *   7  CUDA-core GEMMs on seeded operands against a host sum: per case the
+ *      kind (0 FP64, 1 small products in FP64, 2 in FP32), the terms of a dot
+ *      product and max |C - C_host| / (|alpha| sum |a b| + |beta c0|) */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

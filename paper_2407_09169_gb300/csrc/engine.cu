@@ -265,14 +265,32 @@ void Engine::gemm64(int M, int N, int K, int outer, int inner, double alpha, Mat
   gemm_f64(cur(), M, N, K, outer, inner, alpha, A, B, beta, C, lane_ws_[lane_], ws_elems_);
 }
 
+bool Engine::small_in_fp32(int role) const {
+  return tc_mode_[role] >= 0 && (small_fp32_ || (small_sketch_fp32_ && role != GEMM_STATE && role != GEMM_MIX));
+}
+
+void Engine::gemm_sum(int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B, OutView C,
+                      const SumPieces& P, int role) {
+  if (small_gemm_fits(M, N, K, outer, inner)) {
+    TimeScope ts(timer_, TM_SMALL, cur(), 2.0 * M * (double)N * K * outer * inner * P.n);
+    small_gemm_sum(cur(), small_in_fp32(role), M, N, K, outer, inner, alpha, A, B, 0.0, C, P);
+    return;
+  }
+  for (int p = 0; p < P.n; ++p) {
+    MatView Ap = A, Bp = B;
+    Ap.p += p * P.a;
+    Bp.p += (p & 1) * P.b0 + (p >> 1) * P.b1;
+    gemm(M, N, K, outer, inner, alpha, Ap, Bp, p == 0 ? 0.0 : 1.0, C, role);
+  }
+}
+
 void Engine::gemm(int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B, double beta,
                   OutView C, int role) {
   const int mode = tc_mode_[role];
   if (small_gemm_fits(M, N, K, outer, inner)) {
     // operator-bond contractions: memory-bound, on the CUDA cores
     TimeScope ts(timer_, TM_SMALL, cur(), 2.0 * M * (double)N * K * outer * inner);
-    small_gemm(cur(), mode >= 0 && (small_fp32_ || (small_sketch_fp32_ && role != GEMM_STATE && role != GEMM_MIX)), M, N, K, outer,
-               inner, alpha, A, B, beta, C);
+    small_gemm(cur(), small_in_fp32(role), M, N, K, outer, inner, alpha, A, B, beta, C);
     return;
   }
   if (mode < 0) {
@@ -569,23 +587,26 @@ void Engine::sketch_site(const Term& t, int n, const double* Wn1, double* Wn, co
     gemm(2 * bl, 2 * Ll, br, wr, 1, 1.0, mv(A, br, 1), mv(X1, 2LL * Ll, 1, (long long)br * 2 * Ll), 0.0,
          ov(X2, 2LL * Ll, 1, 4LL * bl * Ll), role);
     // W_n[(w,a)][l] = sum_{s,s',w'} W[w][s*2+s'][w'] X2[w'][(a,s')][(s,l)]
-    const double* Wss = t.op->Wss(n);
-    for (int ss = 0; ss < 4; ++ss) {
-      const int s = ss >> 1, sp = ss & 1;
-      gemm(wl, Ll, wr, bl, 1, 1.0, mv(Wss + (size_t)ss * wl * wr, wr, 1),
-           mv(X2 + (size_t)sp * 2 * Ll + (size_t)s * Ll, 4LL * bl * Ll, 1, 4LL * Ll), ss == 0 ? 0.0 : 1.0,
-           ov(Wn, (long long)bl * Ll, 1, Ll), role);
-    }
+    SumPieces P;
+    P.n = 4;  // p = 2 s + s'
+    P.a = (long long)wl * wr;
+    P.b0 = 2 * Ll;
+    P.b1 = Ll;
+    gemm_sum(wl, Ll, wr, bl, 1, 1.0, mv(t.op->Wss(n), wr, 1), mv(X2, 4LL * bl * Ll, 1, 4LL * Ll),
+             ov(Wn, (long long)bl * Ll, 1, Ll), P, role);
   } else {
     const double* H = t.H(n);
     // X2[a][s][h'][l] = sum_a' A[a][s][a'] X1[(h',a')][s][l]
     gemm(bl, Ll, br, wr, 2, 1.0, mv(A, 2LL * br, 1, 0, br), mv(X1, 2LL * Ll, 1, (long long)br * 2 * Ll, Ll), 0.0,
          ov(X2, 2LL * wr * Ll, 1, Ll, (long long)wr * Ll), role);
-    // W_n[(h,a)][l] = sum_s sum_h' H[h][s][h'] X2[a][s][h'][l], one product per s
-    // accumulated in FP64 (H is shared by every a).
-    for (int s = 0; s < 2; ++s)
-      gemm(wl, Ll, wr, bl, 1, 1.0, mv(H + (size_t)s * wr, 2LL * wr, 1), mv(X2 + (size_t)s * wr * Ll, Ll, 1, 2LL * wr * Ll),
-           s == 0 ? 0.0 : 1.0, ov(Wn, (long long)bl * Ll, 1, Ll), role);
+    // W_n[(h,a)][l] = sum_s sum_h' H[h][s][h'] X2[a][s][h'][l], the two s
+    // added in FP64 (H is shared by every a).
+    SumPieces P;
+    P.n = 2;
+    P.a = wr;
+    P.b0 = (long long)wr * Ll;
+    gemm_sum(wl, Ll, wr, bl, 1, 1.0, mv(H, 2LL * wr, 1), mv(X2, Ll, 1, 2LL * wr * Ll), ov(Wn, (long long)bl * Ll, 1, Ll),
+             P, role);
   }
 }
 

@@ -133,6 +133,16 @@ bool small_gemm_fits(int M, int N, int K, int outer, int inner);
 void small_gemm(cudaStream_t st, bool fp32, int M, int N, int K, int outer, int inner, double alpha, MatView A,
                 MatView B, double beta, OutView C);
 
+// A sum of up to four such products in one launch: C = alpha sum_p A_p B_p +
+// beta C, p = 0 .. n-1, A_p the view A moved by p a elements and B_p the view
+// B moved by (p & 1) b0 + (p >> 1) b1.
+struct SumPieces {
+  int n = 1;
+  long long a = 0, b0 = 0, b1 = 0;
+};
+void small_gemm_sum(cudaStream_t st, bool fp32, int M, int N, int K, int outer, int inner, double alpha, MatView A,
+                    MatView B, double beta, OutView C, const SumPieces& P);
+
 // Thin Householder QR of an m x n row-major matrix (m >= n): Q (m x n,
 // row-major) overwrites Qout.  Computed in float (prec_bits 32) or double;
 // work must hold 2 * m * n + n doubles.  *status != 0 on failure.

@@ -73,6 +73,9 @@ std::vector<double> down(const double* d, size_t n) {
 // which = 3: bias of the tensor-core modes (TF32X3, BF16X3, BF16X6) on positive
 // operands, K in {32, 256, 2048}, with and without a one-k-block cap per
 // accumulator: (mean, max) of the signed relative error (C_tc - C_64) / C_64.
+// which = 7: the CUDA-core GEMMs (FP64, and the small products in FP64 and
+// FP32) against a host sum: per case the kind, the terms of a dot product and
+// max |C - C_host| / (|alpha| sum |a b| + |beta c0|).
 std::vector<double> run_selftest(int which) {
   cudaStream_t st = nullptr;
   std::vector<double> out;
@@ -467,6 +470,99 @@ std::vector<double> run_selftest(int which) {
     cudaEventDestroy(e1);
     out.push_back((double)sms);
     out.push_back((double)blocks);
+  } else if (which == 7) {
+    struct Case {
+      int kind;  // 0: gemm_f64, 1: small products in FP64, 2: in FP32
+      int M, N, K, outer, inner, pieces;
+      bool ta, tb, shared_a;  // shared_a: A does not depend on the outer index
+      double alpha, beta;
+      bool ws;
+    };
+    const Case cases[] = {
+        {0, 1, 1, 1, 1, 1, 1, false, false, false, 1.0, 0.0, false},
+        {0, 40, 40, 80, 1, 1, 1, false, true, false, 1.0, 0.0, false},
+        {0, 136, 136, 272, 1, 1, 1, true, false, false, 1.0, 0.0, false},
+        {0, 33, 73, 31, 3, 2, 1, false, false, false, -1.5, 0.5, false},
+        {0, 272, 136, 4000, 1, 1, 1, false, false, false, 1.0, 1.0, true},
+        {0, 5, 7, 33, 1, 4, 1, true, true, false, 1.0, 0.0, true},
+        {0, 2049, 65, 9, 1, 1, 1, false, false, false, 1.0, 0.0, false},
+        {0, 77, 161, 145, 1, 2, 1, true, true, false, 2.0, 0.0, true},
+        {1, 1, 1, 1, 1, 1, 1, false, false, true, 1.0, 0.0, false},
+        {1, 26, 40, 26, 32, 1, 4, false, false, true, 1.0, 0.0, false},
+        {1, 32, 33, 64, 5, 2, 2, false, false, true, 0.5, 2.0, false},
+        {1, 8, 31, 7, 3, 2, 1, true, false, false, 1.0, 0.0, false},
+        {1, 32, 200, 64, 7, 1, 4, false, true, true, 1.0, 0.0, false},
+        {2, 1, 1, 1, 1, 1, 1, false, false, true, 1.0, 0.0, false},
+        {2, 26, 136, 26, 128, 1, 4, false, false, true, 1.0, 0.0, false},
+        {2, 9, 17, 63, 2, 3, 2, true, false, true, 1.5, 1.0, false},
+        {2, 32, 300, 64, 40, 1, 1, false, false, false, 1.0, 0.0, false}};
+    const size_t ws_elems = (size_t)4 << 20;
+    DBuf ws(ws_elems);
+    unsigned long long seed = 4242;
+    for (const Case& c : cases) {
+      const long long batch = (long long)c.outer * c.inner;
+      const size_t am = (size_t)c.M * c.K, bm = (size_t)c.K * c.N, cm = (size_t)c.M * c.N;
+      const long long na = (c.shared_a ? c.inner : batch) * c.pieces, nb = batch * c.pieces;
+      DBuf A(am * na), B(bm * nb), C0(cm * batch);
+      fill_gaussian(st, A.p, am * na, 1.0, seed++, 1);
+      fill_gaussian(st, B.p, bm * nb, 1.0, seed++, 2);
+      fill_gaussian(st, C0.p, cm * batch, 1.0, seed++, 3);
+      const std::vector<double> ha = down(A.p, am * na), hb = down(B.p, bm * nb), hc = down(C0.p, cm * batch);
+      MatView av, bv;
+      OutView cv;
+      av.p = A.p;
+      av.rs = c.ta ? 1 : c.K;
+      av.cs = c.ta ? c.M : 1;
+      av.si = (long long)am * c.pieces;
+      av.so = c.shared_a ? 0 : av.si * c.inner;
+      bv.p = B.p;
+      bv.rs = c.tb ? 1 : c.N;
+      bv.cs = c.tb ? c.K : 1;
+      bv.si = (long long)bm * c.pieces;
+      bv.so = bv.si * c.inner;
+      cv.p = C0.p;
+      cv.rs = c.N;
+      cv.cs = 1;
+      cv.si = (long long)cm;
+      cv.so = cv.si * c.inner;
+      SumPieces P;
+      P.n = c.pieces;
+      P.a = (long long)am;
+      P.b0 = (long long)bm;
+      P.b1 = 2 * (long long)bm;
+      if (c.kind == 0)
+        gemm_f64(st, c.M, c.N, c.K, c.outer, c.inner, c.alpha, av, bv, c.beta, cv, c.ws ? ws.p : nullptr,
+                 c.ws ? ws_elems : 0);
+      else
+        small_gemm_sum(st, c.kind == 2, c.M, c.N, c.K, c.outer, c.inner, c.alpha, av, bv, c.beta, cv, P);
+      const std::vector<double> got = down(C0.p, cm * batch);
+      double worst = 0.0;
+      for (long long b = 0; b < batch; ++b)
+        for (int m = 0; m < c.M; ++m)
+          for (int n = 0; n < c.N; ++n) {
+            double v = 0.0, mag = 0.0, lost = 0.0;  // compensated sum
+            for (int p = 0; p < c.pieces; ++p) {
+              const double* a = ha.data() + ((c.shared_a ? b % c.inner : b) * c.pieces + p) * am;
+              const double* w = hb.data() + (b * c.pieces + p) * bm;
+              for (int k = 0; k < c.K; ++k) {
+                const double x = a[c.ta ? (size_t)k * c.M + m : (size_t)m * c.K + k];
+                const double y = w[c.tb ? (size_t)n * c.K + k : (size_t)k * c.N + n];
+                const double t = x * y - lost, s = v + t;
+                lost = (s - v) - t;
+                v = s;
+                mag += std::fabs(x * y);
+              }
+            }
+            const size_t e = (size_t)b * cm + (size_t)m * c.N + n;
+            const double ref = c.alpha * v + c.beta * hc[e];
+            const double scale = std::fabs(c.alpha) * mag + std::fabs(c.beta * hc[e]);
+            const double d = std::fabs(got[e] - ref) / scale;
+            worst = d > worst || std::isnan(d) ? d : worst;
+          }
+      out.push_back((double)c.kind);
+      out.push_back((double)c.K * c.pieces);
+      out.push_back(worst);
+    }
   } else {
     cudaFree(err);
     throw std::runtime_error("EINVAL: unknown selftest");

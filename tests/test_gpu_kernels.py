@@ -143,3 +143,20 @@ def test_fp64_throughput_probe():
     dfma, dmma, sms, blocks = v[:4]
     print(f"\nFP64: DFMA {dfma:.3f} TFLOP/s, DMMA {dmma:.3f} TFLOP/s on {int(sms)} SMs ({int(blocks)} blocks)")
     assert 0.05 < dfma < 2.0 and 0.05 < dmma < 2.0
+
+
+CUDA_CORE_CASES = ([0] * 8 + [1] * 5 + [2] * 4)
+
+
+def test_cuda_core_gemms_against_host_sum():
+    """The FP64 GEMM and the small products (edges of the tiles, one-element
+    products, K splits over the warps and over the grid, up to four summed
+    pieces, A shared by the outer batch or not, transposed operands, alpha and
+    beta).  A sum of t terms in any order is within t u of sum |a b|, plus the
+    scaling and the beta term (4 u); in FP32 the operands round too (2 u each)
+    and the partial sums of the warps meet in FP64."""
+    v = np.array(pkg.qtt_selftest(7)[:-1]).reshape(-1, 3)
+    assert [int(k) for k in v[:, 0]] == CUDA_CORE_CASES
+    for kind, terms, err in v:
+        u = 2.0 ** -24 if kind == 2 else 2.0 ** -53
+        assert err <= (terms + 8) * u, (kind, terms, err)
