@@ -2,12 +2,28 @@
 // path for every core contraction, and by all paths for the small FP64 Gram
 // matrices of the SVD truncation sweep.
 //
-// Tile 64 x 64 x 16, 256 threads, 4 x 4 outputs per thread spread with
-// stride 16 so that a warp's shared-memory reads are conflict-free.  The
-// operands are read through general (row, column, batch) strides so that
-// every reshape / transpose of the contraction is a view, not a copy.
-// Split-K writes partial tiles to a workspace that a second kernel reduces
-// in a fixed order (deterministic).
+// FP64 issues at two FMAs per clock per SM: a warp FMA holds its scheduler for
+// 64 clocks, with one lane active as with 32, while loads, shared-memory
+// reads and address arithmetic are almost free beside it.  So the kernel is
+// shaped by two things only: no masked FMAs, and equal numbers of FMAs on the
+// 608 schedulers.  A block of 8 warps computes TM x 8 RN outputs: a warp holds
+// 4 rows x 8 RN columns (lane: one row, RN columns 8 apart), TM / 4 warps cover
+// the rows and the K range is dealt over the 32 / TM groups of warps, whose
+// partial sums meet in shared memory.  Column counts of the bonds used
+// (40, 72, 128, 136: 5, 9, 16 = 8 + 8, 17 = 9 + 8 groups of 8) fit RN <= 9 with
+// little or no waste, where a 64 x 64 tile masks 38 to 47% of its FMAs at 40
+// and 72 columns; TM = 4, 8 and 16 spread the bond-sized products (136 x 136)
+// over all SMs in one launch, where 16 x 16 tiles gave 81 blocks and a K split
+// over the grid needs a reduction launch.  That one remains for products with
+// few outputs and a long K (the range product 272 x 136 x 16384).  Before and
+// after: step of 20 sites chi 32 15.3 -> 10.0 ms, of 30 sites chi 64 44.5 ->
+// 35.7; untruncated step of 10 sites 1.31 -> 0.40; truncation backward of 40
+// sites chi 128 13.6 -> 11.5; 40 sites chi 128 BF16X10 (its Grams) 57.1 -> 55.1.
+//
+// The operands are read through general (row, column, batch) strides so that
+// every reshape / transpose of the contraction is a view, not a copy: chunks
+// of 32 k are loaded into registers while the chunk before is multiplied,
+// along whichever index is contiguous.  Sums are in a fixed order.
 #include <algorithm>
 
 #include "kernels.cuh"
@@ -15,86 +31,104 @@
 namespace qtt {
 
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int NT = 256, KC = 32;
 
+template <int TM, int RN>
 __global__ void __launch_bounds__(NT) gemm_f64_kernel(int M, int N, int K, int inner, int splitk, int kchunk,
-                                                      double alpha, MatView A, MatView B, double beta,
-                                                      OutView C, double* ws) {
+                                                      double alpha, MatView A, MatView B, double beta, OutView C,
+                                                      double* ws) {
+  constexpr int TN = 8 * RN, KS = 32 / TM, LA = TM + 1, LB = TN + 1;
+  constexpr int NA = (TM * KC + NT - 1) / NT, NB = TN * KC / NT;
   pdl_trigger();
   pdl_wait();
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM;
+  __shared__ double smem[KC * (LA + LB)];
+  double* As = smem;            // [KC][LA]
+  double* Bs = smem + KC * LA;  // [KC][LB]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n0 = blockIdx.x * TN, m0 = blockIdx.y * TM;
   const int z = blockIdx.z;
-  const int b = z / splitk, ks = z - b * splitk;
+  const int b = z / splitk, sk = z - b * splitk;
   const int bo = b / inner, bi = b - bo * inner;
   const double* Ap = A.p + bo * A.so + bi * A.si;
   const double* Bp = B.p + bo * B.so + bi * B.si;
-  const int k0 = ks * kchunk;
-  const int k1 = min(K, k0 + kchunk);
+  const int k0 = sk * kchunk, k1 = min(K, k0 + kchunk);
   const bool a_mfast = (A.rs < 0 ? -A.rs : A.rs) <= (A.cs < 0 ? -A.cs : A.cs);
   const bool b_nfast = (B.cs < 0 ? -B.cs : B.cs) <= (B.rs < 0 ? -B.rs : B.rs);
-  double acc[4][4];
+  const int wm = warp % (TM / 4), ks = warp / (TM / 4);
+  const int row = 4 * wm + (lane >> 3), col = lane & 7;
+  const bool rows_live = m0 + 4 * wm < M;  // warp-uniform: a warp with no rows adds no FMAs
+  double acc[RN], ra[NA], rb[NB];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  for (int j = 0; j < RN; ++j) acc[j] = 0.0;
 
-  for (int kt = k0; kt < k1; kt += BK) {
+  auto fetch = [&](int kt) {
 #pragma unroll
-    for (int q = 0; q < (BM * BK) / NT; ++q) {
-      const int idx = tid + q * NT;
-      int mm, kk;
-      if (a_mfast) { mm = idx % BM; kk = idx / BM; } else { kk = idx % BK; mm = idx / BK; }
+    for (int q = 0; q < NA; ++q) {
+      const int x = tid + q * NT;
+      const int kk = a_mfast ? x / TM : x % KC, mm = a_mfast ? x % TM : x / KC;
       const int gm = m0 + mm, gk = kt + kk;
-      As[kk][mm] = (gm < M && gk < k1) ? Ap[(long long)gm * A.rs + (long long)gk * A.cs] : 0.0;
+      ra[q] = (x < TM * KC && gm < M && gk < k1) ? Ap[(long long)gm * A.rs + (long long)gk * A.cs] : 0.0;
     }
 #pragma unroll
-    for (int q = 0; q < (BN * BK) / NT; ++q) {
-      const int idx = tid + q * NT;
-      int nn, kk;
-      if (b_nfast) { nn = idx % BN; kk = idx / BN; } else { kk = idx % BK; nn = idx / BK; }
+    for (int q = 0; q < NB; ++q) {
+      const int x = tid + q * NT;
+      const int kk = b_nfast ? x / TN : x % KC, nn = b_nfast ? x % TN : x / KC;
       const int gn = n0 + nn, gk = kt + kk;
-      Bs[kk][nn] = (gn < N && gk < k1) ? Bp[(long long)gk * B.rs + (long long)gn * B.cs] : 0.0;
+      rb[q] = (gn < N && gk < k1) ? Bp[(long long)gk * B.rs + (long long)gn * B.cs] : 0.0;
+    }
+  };
+  if (k0 < k1) fetch(k0);
+  for (int kt = k0; kt < k1; kt += KC) {
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int x = tid + q * NT;
+      const int kk = a_mfast ? x / TM : x % KC, mm = a_mfast ? x % TM : x / KC;
+      if (x < TM * KC) As[kk * LA + mm] = ra[q];
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int x = tid + q * NT;
+      const int kk = b_nfast ? x / TN : x % KC, nn = b_nfast ? x % TN : x / KC;
+      Bs[kk * LB + nn] = rb[q];
     }
     __syncthreads();
+    if (kt + KC < k1) fetch(kt + KC);  // in flight during the multiplication
+    const int kend = min(KC, k1 - kt);
+    if (rows_live) {
+#pragma unroll 4
+      for (int kk = ks; kk < kend; kk += KS) {
+        const double a = As[kk * LA + row];
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      double a[4], bb[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < RN; ++j) acc[j] = fma(a, Bs[kk * LB + col + 8 * j], acc[j]);
+      }
     }
     __syncthreads();
   }
-  if (ws) {
-    double* W = ws + ((long long)b * splitk + ks) * (long long)M * N;
+  double* W = ws ? ws + ((long long)b * splitk + sk) * (long long)M * N : nullptr;
+  double* Cp = C.p + bo * C.so + bi * C.si;
+  auto put = [&](int gm, int gn, double v) {
+    if (gm >= M || gn >= N) return;
+    if (W) {
+      W[(long long)gm * N + gn] = v;
+    } else {
+      double* c = Cp + (long long)gm * C.rs + (long long)gn * C.cs;
+      *c = (beta == 0.0) ? alpha * v : alpha * v + beta * (*c);
+    }
+  };
+  if (KS == 1) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int gm = m0 + ty + 16 * i, gn = n0 + tx + 16 * j;
-        if (gm < M && gn < N) W[(long long)gm * N + gn] = acc[i][j];
-      }
+    for (int j = 0; j < RN; ++j) put(m0 + row, n0 + col + 8 * j, acc[j]);
   } else {
-    double* Cp = C.p + bo * C.so + bi * C.si;
+    // [KS][TM][TN] partial sums: 32 TN doubles, within the operand buffers
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int j = 0; j < RN; ++j) smem[(ks * TM + row) * TN + col + 8 * j] = acc[j];
+    __syncthreads();
+    for (int x = tid; x < TM * TN; x += NT) {
+      double v = smem[x];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int gm = m0 + ty + 16 * i, gn = n0 + tx + 16 * j;
-        if (gm < M && gn < N) {
-          double* c = Cp + (long long)gm * C.rs + (long long)gn * C.cs;
-          *c = (beta == 0.0) ? alpha * acc[i][j] : alpha * acc[i][j] + beta * (*c);
-        }
-      }
+      for (int q = 1; q < KS; ++q) v += smem[q * TM * TN + x];
+      put(m0 + x / TN, n0 + x % TN, v);
+    }
   }
 }
 
@@ -131,41 +165,6 @@ __global__ void scale_out_kernel(int M, int N, int inner, int batch, double beta
     *c = (beta == 0.0) ? 0.0 : beta * (*c);
   }
 }
-// Products whose 64 x 64 tile grid is too small for the GPU (the bond-sized
-// FP64 products: right Grams of the truncation, 136 x 136 x 272) otherwise
-// need a K split and a reduction launch.  16 x 16 output tiles give them
-// enough blocks instead, each thread summing its whole dot product (K in
-// chunks of 32 staged through shared memory), with the strided views and
-// alpha / beta of gemm_f64.
-__global__ void __launch_bounds__(256) gemm_f64_t16_kernel(int M, int N, int K, int inner, double alpha, MatView A,
-                                                           MatView B, double beta, OutView C) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ double As[16][33], Bs[32][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * 16, n0 = blockIdx.x * 16;
-  const int b = blockIdx.z, bo = b / inner, bi = b - bo * inner;
-  const double* Ap = A.p + bo * A.so + bi * A.si;
-  const double* Bp = B.p + bo * B.so + bi * B.si;
-  double acc = 0.0;
-  for (int k0 = 0; k0 < K; k0 += 32) {
-    for (int e = threadIdx.x; e < 512; e += 256) {
-      const int rr = e >> 5, kk = e & 31;  // As[rr][kk] = A(m0 + rr, k0 + kk)
-      As[rr][kk] = (m0 + rr < M && k0 + kk < K) ? Ap[(long long)(m0 + rr) * A.rs + (long long)(k0 + kk) * A.cs] : 0.0;
-      const int kb = e >> 4, cc = e & 15;  // Bs[kb][cc] = B(k0 + kb, n0 + cc)
-      Bs[kb][cc] = (k0 + kb < K && n0 + cc < N) ? Bp[(long long)(k0 + kb) * B.rs + (long long)(n0 + cc) * B.cs] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) acc = fma(As[ty][kk], Bs[kk][tx], acc);
-    __syncthreads();
-  }
-  if (m0 + ty < M && n0 + tx < N) {
-    double* c = C.p + bo * C.so + bi * C.si + (long long)(m0 + ty) * C.rs + (long long)(n0 + tx) * C.cs;
-    *c = (beta == 0.0) ? alpha * acc : alpha * acc + beta * (*c);
-  }
-}
-
 // One Newton-Schulz step of an almost-orthonormal Q (m x n, row-major):
 // out = Q (3 I - Q^T Q) / 2, in two launches.  FP64 issues at two operations
 // per clock per SM, so both are sized to one wave of at most 152 blocks with
@@ -259,16 +258,82 @@ void splitk_reduce(cudaStream_t st, int M, int N, int inner, int splitk, int bat
              (const double*)ws, beta, C);
 }
 
-int gemm_split_k(int M, int N, int K, int batch) {
-  const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN) * batch;
-  if (tiles >= 152 || K < 2 * BK) return 1;
-  // FP64 issues at two operations per clock per SM: spread small products
-  // over about two waves of SMs, down to one k-tile per split
-  long long s = (304 + tiles - 1) / tiles;
-  s = s < (K / BK) ? s : (K / BK);
-  if (s > 64) s = 64;
-  return s < 1 ? 1 : (int)s;
+namespace {
+// Tile (TM rows, RN groups of 8 columns) and grid K split of a product, by the
+// clocks of the SM with the most blocks: per block its share of the warp FMAs
+// (two warps a scheduler, 64 clocks each) and what does not overlap with them
+// (about 2000 clocks of load latency and epilogue, 100 per chunk of K).  A
+// split over the grid adds its reduction launch and the partial tiles.
+struct F64Plan {
+  int tm = 32, rn = 9, split = 1, kchunk = 0;
+};
+F64Plan search_f64(int M, int N, int K, long long batch, size_t ws_elems) {
+  F64Plan best;
+  double tbest = 1e300;
+  const int smax = (int)std::min<long long>(64, (K + KC - 1) / KC);
+  for (int s = 1; s <= smax; s *= 2) {
+    if (s > 1 && ((size_t)s * batch * (size_t)M * N > ws_elems || s * batch > 65535)) break;
+    int kchunk = (K + s - 1) / s;
+    if (s > 1) kchunk = (kchunk + KC - 1) / KC * KC;
+    const int sr = (K + kchunk - 1) / kchunk;
+    for (int tm = 4; tm <= 32; tm *= 2) {
+      if ((M + tm - 1) / tm > 65535) continue;
+      for (int rn = 1; rn <= 9; ++rn) {
+        const long long tiles = (long long)((M + tm - 1) / tm) * ((N + 8 * rn - 1) / (8 * rn)) * batch * sr;
+        const int ks = 32 / tm;
+        const double block = (double)((kchunk + ks - 1) / ks) * rn * 128.0 + (kchunk + KC - 1) / KC * 100.0;
+        double t = (double)((tiles + 151) / 152) * block + 2000.0;
+        if (sr > 1) t += 6000.0 + (2.0 * sr + 1.0) * 8.0 * M * N * (double)batch / 2000.0;
+        if (t < tbest) {
+          tbest = t;
+          best.tm = tm;
+          best.rn = rn;
+          best.split = sr;
+          best.kchunk = kchunk;
+        }
+      }
+    }
+  }
+  return best;
 }
+
+// The search is a few hundred evaluations, so each host thread keeps the plans
+// of the shapes it met (a fixed table; a plan depends on nothing else).
+F64Plan plan_f64(int M, int N, int K, long long batch, size_t ws_elems) {
+  struct Entry {
+    int M = 0, N = 0, K = 0;
+    long long batch = 0;
+    size_t ws = 0;
+    F64Plan plan;
+  };
+  thread_local Entry table[512];
+  const unsigned long long key = ((((unsigned long long)M * 1000003ull + N) * 1000003ull + K) * 1000003ull + batch) ^ ws_elems;
+  Entry& e = table[(key * 0x9E3779B97F4A7C15ull) >> 55];
+  if (e.M != M || e.N != N || e.K != K || e.batch != batch || e.ws != ws_elems) {
+    e.M = M;
+    e.N = N;
+    e.K = K;
+    e.batch = batch;
+    e.ws = ws_elems;
+    e.plan = search_f64(M, N, K, batch, ws_elems);
+  }
+  return e.plan;
+}
+
+template <int TM>
+void launch_f64(cudaStream_t st, int rn, dim3 grid, int M, int N, int K, int inner, int splitk, int kchunk, double alpha,
+                MatView A, MatView B, double beta, OutView C, double* ws) {
+#define QTT_F64(RN_)                                                                                               \
+  case RN_:                                                                                                        \
+    launch_pdl(gemm_f64_kernel<TM, RN_>, grid, dim3(NT), 0, st, M, N, K, inner, splitk, kchunk, alpha, A, B, beta, \
+               C, ws);                                                                                             \
+    break;
+  switch (rn) {
+    QTT_F64(1) QTT_F64(2) QTT_F64(3) QTT_F64(4) QTT_F64(5) QTT_F64(6) QTT_F64(7) QTT_F64(8) QTT_F64(9)
+  }
+#undef QTT_F64
+}
+}  // namespace
 
 void gemm_f64(cudaStream_t st, int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B,
               double beta, OutView C, double* ws, size_t ws_elems) {
@@ -295,45 +360,18 @@ void gemm_f64(cudaStream_t st, int M, int N, int K, int outer, int inner, double
     scale_out_kernel<<<blocks, 256, 0, st>>>(M, N, inner, batch, beta, C);
     return;
   }
-  int splitk = gemm_split_k(M, N, K, batch);
-  {
-    const long long t16 = (long long)((M + 15) / 16) * ((N + 15) / 16) * batch;
-    if (splitk > 1 && t16 >= 64 && K <= 2048 && batch <= 65535) {
-      count_launches(1);
-      launch_pdl(gemm_f64_t16_kernel, dim3((N + 15) / 16, (M + 15) / 16, batch), dim3(256), 0, st, M, N, K, inner, alpha,
-                 A, B, beta, C);
-      return;
-    }
+  const F64Plan p = plan_f64(M, N, K, batch, ws ? ws_elems : 0);
+  const dim3 grid((unsigned)((N + 8 * p.rn - 1) / (8 * p.rn)), (unsigned)((M + p.tm - 1) / p.tm),
+                  (unsigned)(batch * p.split));
+  double* w = p.split > 1 ? ws : nullptr;
+  count_launches(p.split == 1 ? 1 : 2);
+  switch (p.tm) {
+    case 4: launch_f64<4>(st, p.rn, grid, M, N, K, inner, p.split, p.kchunk, alpha, A, B, beta, C, w); break;
+    case 8: launch_f64<8>(st, p.rn, grid, M, N, K, inner, p.split, p.kchunk, alpha, A, B, beta, C, w); break;
+    case 16: launch_f64<16>(st, p.rn, grid, M, N, K, inner, p.split, p.kchunk, alpha, A, B, beta, C, w); break;
+    default: launch_f64<32>(st, p.rn, grid, M, N, K, inner, p.split, p.kchunk, alpha, A, B, beta, C, w); break;
   }
-  if (splitk > 1 && (ws == nullptr || (size_t)splitk * batch * (size_t)M * N > ws_elems)) splitk = 1;
-  int kchunk = (K + splitk - 1) / splitk;
-  kchunk = ((kchunk + BK - 1) / BK) * BK;
-  splitk = (K + kchunk - 1) / kchunk;
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch * splitk);
-  count_launches(splitk == 1 ? 1 : 2);
-  if (splitk == 1) {
-    launch_pdl(gemm_f64_kernel, grid, dim3(NT), 0, st, M, N, K, inner, 1, kchunk, alpha, A, B, beta, C,
-               (double*)nullptr);
-  } else {
-    launch_pdl(gemm_f64_kernel, grid, dim3(NT), 0, st, M, N, K, inner, splitk, kchunk, alpha, A, B, beta, C, ws);
-    const long long total = (long long)M * N * batch;
-    int blocks = (int)((total + 255) / 256);
-    if (blocks > 4096) blocks = 4096;
-    launch_pdl(splitk_reduce_kernel, dim3((unsigned)blocks), dim3(256), 0, st, M, N, inner, splitk, batch, alpha,
-             (const double*)ws, beta, C);
-  }
-}
-
-void gemm_f64_tiles16(cudaStream_t st, int M, int N, int K, double alpha, MatView A, MatView B, double beta,
-                      OutView C) {
-  if (M <= 0 || N <= 0) return;
-  if (K <= 0 || M > 65535 * 16) {  // empty contraction, or more row tiles than grid.y holds
-    gemm_f64(st, M, N, K, 1, 1, alpha, A, B, beta, C, nullptr, 0);
-    return;
-  }
-  count_launches(1);
-  launch_pdl(gemm_f64_t16_kernel, dim3((N + 15) / 16, (M + 15) / 16, 1), dim3(256), 0, st, M, N, K, 1, alpha, A, B,
-             beta, C);
+  if (p.split > 1) splitk_reduce(st, M, N, inner, p.split, batch, alpha, ws, beta, C);
 }
 
 void newton_schulz_step(cudaStream_t st, int m, int n, const double* Q, double* G, double* out) {
