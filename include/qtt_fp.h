@@ -350,7 +350,9 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *      the number of blocks
  *   7  CUDA-core GEMMs on seeded operands against a host sum: per case the
  *      kind (0 FP64, 1 small products in FP64, 2 in FP32), the terms of a dot
- *      product and max |C - C_host| / (|alpha| sum |a b| + |beta c0|) */
+ *      product and max |C - C_host| / (|alpha| sum |a b| + |beta c0|)
+ *   8  FP64 eigensolver on a batch of 14 problems of different sizes, the
+ *      leading k columns: the three values of 2 per problem */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

@@ -160,3 +160,13 @@ def test_cuda_core_gemms_against_host_sum():
     for kind, terms, err in v:
         u = 2.0 ** -24 if kind == 2 else 2.0 ** -53
         assert err <= (terms + 8) * u, (kind, terms, err)
+
+
+def test_batched_eigensolver_of_mixed_sizes():
+    """One pass over problems of 1 to 193 rows: the edges of the leaves (12
+    rows) and of the merge levels, problems with fewer levels than the largest,
+    partial sets of vectors, and rank-deficient matrices (rotated and
+    negligible poles).  The bound is the eigensolver's own, 1e-12."""
+    v = np.array(pkg.qtt_selftest(8)[:-1]).reshape(-1, 3)
+    assert v.shape[0] == 14
+    assert (v[:, :2] < 1e-12).all() and (v[:, 2] == 0).all(), v
