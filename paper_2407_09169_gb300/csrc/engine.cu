@@ -179,6 +179,7 @@ Engine::~Engine() {
   for (cudaGraph_t& g : graph_tmpl_)
     if (g) cudaGraphDestroy(g);
   for (void* a : allocs_) cudaFree(a);
+  if (obs_buf_) cudaFree(obs_buf_);
   for (void* w : pack_ws_)
     if (w) cudaFree(w);
   for (int l = 1; l < kLanes; ++l) {
@@ -533,9 +534,10 @@ void Engine::init() {
   QTT_CUDA(cudaMemsetAsync(status_, 0, sizeof(int) * 4, st_));
   if (mref_) {  // the reference starts from the initial <Phi_a>(x)
     const size_t Mx = (size_t)1 << (p_.bits[2] + p_.bits[3] + p_.bits[4]);
-    double* tmp3 = (double*)dalloc(3 * Mx * sizeof(double));
-    means_dev(tmp3);
-    QTT_CUDA(cudaMemcpyAsync(mref_, tmp3 + Mx, 2 * Mx * sizeof(double), cudaMemcpyDeviceToDevice, st_));
+    Scratch s(*this, chain_dense_bytes(3 * Mx));
+    const double* fields = means_dev((double*)s.p);
+    QTT_CUDA(cudaMemcpyAsync(mref_, fields + Mx, 2 * Mx * sizeof(double), cudaMemcpyDeviceToDevice, st_));
+    QTT_CUDA(cudaStreamSynchronize(st_));
   }
   QTT_CUDA(cudaStreamSynchronize(st_));
 }
@@ -1084,46 +1086,62 @@ void Engine::scalars(double out[13]) {
   out[12] = n2;  // sum of f^2 over every grid cell
 }
 
+Engine::Scratch::Scratch(Engine& e, size_t bytes) : eng(e) {
+  if (bytes <= kObsKeep && !e.obs_busy_) {
+    if (bytes > e.obs_bytes_) {
+      if (e.obs_buf_) {
+        QTT_CUDA(cudaStreamSynchronize(e.st_));
+        QTT_CUDA(cudaFree(e.obs_buf_));
+      }
+      e.obs_buf_ = nullptr;
+      e.obs_bytes_ = 0;
+      QTT_CUDA(cudaMalloc(&e.obs_buf_, bytes));
+      e.obs_bytes_ = bytes;
+    }
+    e.obs_busy_ = true;
+    kept = true;
+    p = (unsigned char*)e.obs_buf_;
+  } else {
+    QTT_CUDA(cudaMalloc(&p, bytes));
+  }
+}
+
+Engine::Scratch::~Scratch() {
+  if (kept) eng.obs_busy_ = false;
+  else if (p) cudaFree(p);
+}
+
+size_t Engine::chain_dense_bytes(size_t rows) { return sizeof(double) * (rows + 16) * 4; }
+
 void Engine::chain_dense(const DevMps& f, int n0, const double* head, int head_rows, double* out) {
   size_t rows = head_rows;
   for (int n = n0; n < N_; ++n) rows *= 2;
-  double* d = nullptr;
-  QTT_CUDA(cudaMalloc(&d, sizeof(double) * rows));
-  try {
-    chain_dense_dev(f, n0, head, head_rows, d);
-    QTT_CUDA(cudaMemcpyAsync(out, d, sizeof(double) * rows, cudaMemcpyDeviceToHost, st_));
-    QTT_CUDA(cudaStreamSynchronize(st_));
-  } catch (...) {
-    cudaFree(d);
-    throw;
-  }
-  cudaFree(d);
+  Scratch s(*this, chain_dense_bytes(rows));
+  const double* d = chain_dense_dev(f, n0, head, head_rows, (double*)s.p);
+  QTT_CUDA(cudaMemcpyAsync(out, d, sizeof(double) * rows, cudaMemcpyDeviceToHost, st_));
+  QTT_CUDA(cudaStreamSynchronize(st_));
 }
 
-void Engine::chain_dense_dev(const DevMps& f, int n0, const double* head, int head_rows, double* dout) {
-  // rows = multi-index of the processed sites, columns = open bond; out gets head_rows * 2^(N - n0) values
+const double* Engine::chain_dense_dev(const DevMps& f, int n0, const double* head, int head_rows, double* work) {
+  // rows = multi-index of the processed sites, columns = open bond
   size_t rows = head_rows;
   for (int n = n0; n < N_; ++n) rows *= 2;
-  double* a = nullptr;
-  double* b = nullptr;
-  QTT_CUDA(cudaMalloc(&a, sizeof(double) * (rows * 1 + 16) * 2));
-  QTT_CUDA(cudaMalloc(&b, sizeof(double) * (rows * 1 + 16) * 2));
   // buffer bound: rows_so_far * bond <= head_rows * 2^(N-n0) when bonds follow the structural profile
+  double* a = work;
+  double* b = work + (rows + 16) * 2;
   size_t R = head_rows;
   int bond = f.b[n0];
-  QTT_CUDA(cudaMemcpyAsync(a, head, sizeof(double) * R * bond, cudaMemcpyDeviceToDevice, st_));
+  const double* cur = head;
   for (int n = n0; n < N_; ++n) {
     const int br = f.b[n + 1];
-    gemm64((int)R, 2 * br, bond, 1, 1, 1.0, mv(a, bond, 1), mv(f.core(n), 2LL * br, 1), 0.0, ov(b, 2LL * br, 1));
+    gemm64((int)R, 2 * br, bond, 1, 1, 1.0, mv(cur, bond, 1), mv(f.core(n), 2LL * br, 1), 0.0, ov(a, 2LL * br, 1));
+    cur = a;
     std::swap(a, b);
     R *= 2;
     bond = br;
   }
   QTT_CUDA(cudaGetLastError());
-  QTT_CUDA(cudaMemcpyAsync(dout, a, sizeof(double) * R, cudaMemcpyDeviceToDevice, st_));
-  QTT_CUDA(cudaStreamSynchronize(st_));
-  cudaFree(a);
-  cudaFree(b);
+  return cur;
 }
 
 void Engine::dense(double* out) {
@@ -1131,34 +1149,31 @@ void Engine::dense(double* out) {
   chain_dense(f_, 0, obsA_, 1, out);
 }
 
-void Engine::means_dev(double* dout) {
+const double* Engine::means_dev(double* work) {
+  // the three weight environments as the three heads of one chain; rows (w, x)
   const int b = D_[kphi_];
-  const size_t Mx = (size_t)1 << (p_.bits[2] + p_.bits[3] + p_.bits[4]);
-  const Chain fc = f_.chain();
-  for (int w = 0; w < 3; ++w) {
-    left_weight_env(st_, fc, wphi_[w].chain(), kphi_, max_bond_, envout_, b, envw_);
-    chain_dense_dev(f_, kphi_, envout_, 1, dout + w * Mx);
+  if (max_bond_ <= 1600) {
+    left_weight_envs(st_, f_.chain(), wchains_dev_, 3, kphi_, max_bond_, envout_, b, b);
+  } else {  // environments beyond the shared memory of the batched kernel
+    for (int w = 0; w < 3; ++w)
+      left_weight_env(st_, f_.chain(), wphi_[w].chain(), kphi_, max_bond_, envout_ + (size_t)w * b, b, envw_);
   }
+  return chain_dense_dev(f_, kphi_, envout_, 3, work);
 }
 
 void Engine::error_sample(double* out) {
   if (!mref_) throw std::runtime_error("EINVAL: the error measures need moment_ref = 1");
   const size_t Mx = (size_t)1 << (p_.bits[2] + p_.bits[3] + p_.bits[4]);
-  double* fields = nullptr;
-  QTT_CUDA(cudaMalloc(&fields, 3 * Mx * sizeof(double)));
   double acc[5] = {0, 0, 0, 0, 0};
-  try {
-    means_dev(fields);
+  {
+    Scratch s(*this, chain_dense_bytes(3 * Mx));
+    const double* fields = means_dev((double*)s.p);
     QTT_CUDA(cudaMemsetAsync(errs_, 0, 5 * sizeof(double), st_));
     error_sums(st_, fields, mref_, Mx, errs_);
     QTT_CUDA(cudaGetLastError());
     QTT_CUDA(cudaMemcpyAsync(acc, errs_, sizeof(acc), cudaMemcpyDeviceToHost, st_));
     QTT_CUDA(cudaStreamSynchronize(st_));
-  } catch (...) {
-    cudaFree(fields);
-    throw;
   }
-  cudaFree(fields);
   const double n = (double)Mx, a1 = acc[3] / n, a2 = acc[4] / n;
   out[0] = a1 - 0.5;
   out[1] = a2 - 0.5;
@@ -1169,28 +1184,23 @@ void Engine::error_sample(double* out) {
 }
 
 void Engine::means(double* out) {
-  const int b = D_[kphi_];
   const size_t Mx = (size_t)1 << (p_.bits[2] + p_.bits[3] + p_.bits[4]);
-  const Chain fc = f_.chain();
-  for (int w = 0; w < 3; ++w) {
-    left_weight_env(st_, fc, wphi_[w].chain(), kphi_, max_bond_, envout_, b, envw_);
-    chain_dense(f_, kphi_, envout_, 1, out + w * Mx);
-  }
+  Scratch s(*this, chain_dense_bytes(3 * Mx));
+  const double* d = means_dev((double*)s.p);
+  QTT_CUDA(cudaMemcpyAsync(out, d, 3 * Mx * sizeof(double), cudaMemcpyDeviceToHost, st_));
+  QTT_CUDA(cudaStreamSynchronize(st_));
 }
 
 void Engine::points(const std::vector<unsigned char>& bits, int npts, double* out) {
-  unsigned char* db = nullptr;
-  double *dout = nullptr, *work = nullptr;
-  QTT_CUDA(cudaMalloc(&db, bits.size() + 1));
-  QTT_CUDA(cudaMalloc(&dout, sizeof(double) * npts));
-  QTT_CUDA(cudaMalloc(&work, sizeof(double) * (size_t)npts * 2 * max_bond_));
+  const size_t vb = ((size_t)npts * sizeof(double) + 255) & ~(size_t)255;
+  Scratch s(*this, vb + bits.size() + 256);
+  double* dout = (double*)s.p;
+  unsigned char* db = s.p + vb;
   QTT_CUDA(cudaMemcpyAsync(db, bits.data(), bits.size(), cudaMemcpyHostToDevice, st_));
-  eval_points(st_, f_.chain(), npts, db, max_bond_, dout, work);
+  eval_points(st_, f_.chain(), npts, db, max_bond_, dout);
+  QTT_CUDA(cudaGetLastError());
   QTT_CUDA(cudaMemcpyAsync(out, dout, sizeof(double) * npts, cudaMemcpyDeviceToHost, st_));
   QTT_CUDA(cudaStreamSynchronize(st_));
-  cudaFree(db);
-  cudaFree(dout);
-  cudaFree(work);
 }
 
 double Engine::overlap(const Engine& o) {

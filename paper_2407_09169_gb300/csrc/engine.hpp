@@ -204,9 +204,10 @@ class Engine {
   Term term_dense(int slot, const DevOp* op, const DevMps* f, double scale) const;
   Term term_mix(const DevMps* f, const double* hf, double scale) const;
   void chain_dense(const DevMps& f, int n0, const double* head, int head_rows, double* out);
-  // the same into device memory (dout holds head_rows * 2^(N - n0) doubles)
-  void chain_dense_dev(const DevMps& f, int n0, const double* head, int head_rows, double* dout);
-  void means_dev(double* dout);  // <1>, <Phi_1>, <Phi_2> over x into device memory
+  // the same left on the device: work holds chain_dense_bytes(head_rows * 2^(N - n0)), the result is in it
+  const double* chain_dense_dev(const DevMps& f, int n0, const double* head, int head_rows, double* work);
+  static size_t chain_dense_bytes(size_t rows);
+  const double* means_dev(double* work);  // <1>, <Phi_1>, <Phi_2> over x (chain_dense_bytes(3 Mx) of work)
   void moment_ref_step();        // one RK2 step of the first-moment reference (moment_ref)
   // adjoint (adjoint.cu)
   void grad_setup();
@@ -218,6 +219,23 @@ class Engine {
   void sandwich_acc(const DevMps& a, const Term& t, double w, double* acc);
   void grad_terms(const DevMps& a, const DevMps& f, const double* hf, double w);
   void set_step_counter(unsigned long long s);
+
+  // Device scratch of one observable call: the engine's kept buffer up to
+  // kObsKeep bytes (it grows with the requests and goes with the engine), an
+  // allocation of its own above that.
+  static constexpr size_t kObsKeep = (size_t)64 << 20;
+  struct Scratch {
+    Engine& eng;
+    unsigned char* p = nullptr;
+    bool kept = false;
+    Scratch(Engine& e, size_t bytes);
+    ~Scratch();
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+  };
+  void* obs_buf_ = nullptr;
+  size_t obs_bytes_ = 0;
+  bool obs_busy_ = false;
 
   Params p_;
   Model model_;

@@ -81,32 +81,96 @@ struct Chain {
   int n;
 };
 
+// Points a block of the point evaluation carries, and its shared memory.  FP64
+// issue bounds it (one FMA per point and core entry of its bit), so few points
+// go eight to a block, sharing each load of a core between them, once there
+// are enough to fill the SMs that way, and four otherwise; bonds whose rows do
+// not fit take fewer.
+constexpr int kEvalThreads = 256;
+inline size_t eval_points_smem(int pt, int max_bond) {
+  return ((size_t)2 * pt * max_bond + (size_t)kEvalThreads * pt) * sizeof(double);
+}
+inline int eval_points_per_block(int npts, int max_bond) {
+  int pt = npts > 8 * 304 ? 8 : 4;
+  while (pt > 1 && eval_points_smem(pt, max_bond) > 160 * 1024) pt /= 2;
+  return pt;
+}
+
 #ifdef __CUDACC__
-// f at one grid point, evaluated by one warp: the row vector v (length of the
-// current bond) is carried through the chain, v <- v A_n[:, s_n, :], with s_n
-// the n-th index bit of the point, read by bit(n) (any flag type: bytes or
-// 0/1 doubles).  v and v2 are two scratch rows of max_bond doubles owned by
-// the warp; every entry read has been written first, so the scratch needs no
-// clearing.  Returns the value on every lane.
-template <typename BitFn>
-__device__ __forceinline__ double eval_point_warp(const Chain& f, BitFn bit, double* v, double* v2) {
-  const int lane = threadIdx.x & 31;
-  if (lane == 0) v[0] = 1.0;
-  __syncwarp();
+// f at up to PT grid points, evaluated by one block of kEvalThreads: the row
+// vectors v (length of the current bond) are carried through the chain, v <- v
+// A_n[:, s_n, :], with s_n the n-th index bit of each point, read by bit(p, n)
+// (any flag type: bytes or 0/1 doubles).  A warp takes 32 columns and a part
+// of the rows of a core (the parts' sums meet in shared memory), so a core
+// entry is loaded once for all points of the block and eight are in flight.
+// sm: eval_points_smem(PT, max_bond) bytes.  4096 points of a 30-site chi = 64
+// state with copies take 0.8 ms and 512 points of a 40-site chi = 128 state 0.6.
+// (Before, a warp per point kept its row in global memory, one dependent load
+// and FMA after another: the points, mean fields and scalars of the 30-site
+// state together took 3.3 ms, now 2.3.)
+template <int PT, typename BitFn>
+__device__ __forceinline__ void eval_points_block(const Chain& f, BitFn bit, int npts, int max_bond, double* sm,
+                                                  double* out) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double* v = sm;
+  double* v2 = sm + (size_t)PT * max_bond;
+  double* red = v2 + (size_t)PT * max_bond;
+  for (int p = tid; p < PT; p += kEvalThreads) v[(size_t)p * max_bond] = 1.0;
+  __syncthreads();
   for (int n = 0; n < f.n; ++n) {
     const int bl = f.bond[n], br = f.bond[n + 1];
-    const int s = bit(n) ? 1 : 0;
     const double* A = f.core[n];
-    for (int c = lane; c < br; c += 32) {
-      double acc = 0.0;
-      for (int b = 0; b < bl; ++b) acc += v[b] * A[((size_t)b * 2 + s) * br + c];
-      v2[c] = acc;
+    bool s[PT];
+#pragma unroll
+    for (int p = 0; p < PT; ++p) s[p] = p < npts && bit(p, n);
+    const int chunks = (br + 31) / 32;
+    const int wc = chunks >= 8 ? 8 : chunks > 4 ? 8 : chunks > 2 ? 4 : chunks;  // warps across the columns
+    const int parts = 8 / wc, part = warp / wc;
+    const int b0 = bl * part / parts, b1 = bl * (part + 1) / parts;
+    for (int ch = warp % wc; ch < chunks; ch += wc) {
+      const int c = ch * 32 + lane;
+      double acc[PT];
+#pragma unroll
+      for (int p = 0; p < PT; ++p) acc[p] = 0.0;
+      for (int b = b0; b < b1; b += 4) {
+        double a0[4], a1[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool live = c < br && b + u < b1;
+          a0[u] = live ? A[((size_t)(b + u) * 2) * br + c] : 0.0;
+          a1[u] = live ? A[((size_t)(b + u) * 2 + 1) * br + c] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (b + u >= b1) break;  // warp-uniform
+#pragma unroll
+          for (int p = 0; p < PT; ++p) acc[p] = fma(v[(size_t)p * max_bond + b + u], s[p] ? a1[u] : a0[u], acc[p]);
+        }
+      }
+      if (parts == 1) {
+        if (c < br)
+#pragma unroll
+          for (int p = 0; p < PT; ++p) v2[(size_t)p * max_bond + c] = acc[p];
+      } else {
+#pragma unroll
+        for (int p = 0; p < PT; ++p) red[((size_t)part * PT + p) * (32 * wc) + c] = acc[p];
+      }
     }
-    __syncwarp();
-    for (int c = lane; c < br; c += 32) v[c] = v2[c];
-    __syncwarp();
+    __syncthreads();
+    if (parts > 1) {
+      for (int x = tid; x < PT * br; x += kEvalThreads) {
+        const int p = x / br, c = x - p * br;
+        double t = red[(size_t)p * (32 * wc) + c];
+        for (int q = 1; q < parts; ++q) t += red[((size_t)q * PT + p) * (32 * wc) + c];
+        v2[(size_t)p * max_bond + c] = t;
+      }
+      __syncthreads();
+    }
+    double* t = v;
+    v = v2;
+    v2 = t;
   }
-  return v[0];
+  for (int p = tid; p < npts; p += kEvalThreads) out[p] = v[(size_t)p * max_bond];
 }
 #endif
 
@@ -209,10 +273,8 @@ void left_weight_env(cudaStream_t st, const Chain& f, const Chain& w, int nsites
 void left_weight_envs(cudaStream_t st, const Chain& f, const Chain* wchains_dev, int nw, int nsites, int max_bond,
                       double* out, long long out_stride, int ldo);
 // u[b] = sum over the indices of sites [n0, N) of f(..)[b]: right environment
-// with the all-ones vector.  One block; work holds 2 * max_bond doubles.
+// with the all-ones vector.  One block, a warp per row; work holds 2 * max_bond doubles.
 void right_ones_env(cudaStream_t st, const Chain& f, int n0, int max_bond, double* out, double* work);
-// Evaluates f at npts multi-indices given as bits[p * N + n] (one warp per
-// point); work holds npts * 2 * max_bond doubles.
 // Diagonal cores of the mixing term under the subgrid closures: the x cores
 // of f (the first one replaced by hf, [2][2][b], the conditional means
 // absorbed) times the x cores of the Omega_mix(x) train, site by site as a
@@ -231,8 +293,8 @@ void moment_stage(cudaStream_t st, const double* m0, const double* m, double* ou
 // (N - 1)^2, M1, M2 over the x grid (fields [3][Mx] = <1>, <Phi_1>, <Phi_2>;
 // ref [2][Mx]); acc must be zeroed first.
 void error_sums(cudaStream_t st, const double* fields, const double* ref, size_t Mx, double* acc);
-void eval_points(cudaStream_t st, const Chain& f, int npts, const unsigned char* bits, int max_bond, double* out,
-                 double* work);
+// Evaluates f at npts multi-indices given as bits[p * N + n].
+void eval_points(cudaStream_t st, const Chain& f, int npts, const unsigned char* bits, int max_bond, double* out);
 // flag[0] = 1 if any of the n entries is NaN or infinite.
 void check_finite(cudaStream_t st, const double* p, size_t n, int* flag);
 

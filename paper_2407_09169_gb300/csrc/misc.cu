@@ -220,35 +220,44 @@ __global__ void left_weight_envs_kernel(Chain f, const Chain* __restrict__ wchai
   }
 }
 
-__global__ void right_ones_env_kernel(Chain f, int n0, int max_bond, double* out, double* work) {
+__global__ void __launch_bounds__(1024) right_ones_env_kernel(Chain f, int n0, int max_bond, double* out, double* work) {
   double* R = work;
   double* R2 = work + max_bond;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) R[0] = 1.0;
   __syncthreads();
   for (int n = f.n - 1; n >= n0; --n) {
     const int bl = f.bond[n], br = f.bond[n + 1];
     const double* A = f.core[n];
-    for (int b = threadIdx.x; b < bl; b += blockDim.x) {
-      double acc = 0.0;
-      for (int s = 0; s < 2; ++s)
-        for (int c = 0; c < br; ++c) acc += A[((size_t)b * 2 + s) * br + c] * R[c];
-      R2[b] = acc;
+    for (int b = warp; b < bl; b += 32) {
+      double a0 = 0.0, a1 = 0.0;
+      for (int c = lane; c < br; c += 32) {
+        const double r = R[c];
+        a0 = fma(A[((size_t)b * 2) * br + c], r, a0);
+        a1 = fma(A[((size_t)b * 2 + 1) * br + c], r, a1);
+      }
+      a0 += a1;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+      if (lane == 0) R2[b] = a0;
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < bl; b += blockDim.x) R[b] = R2[b];
-    __syncthreads();
+    double* t = R;
+    R = R2;
+    R2 = t;
   }
   for (int b = threadIdx.x; b < f.bond[n0]; b += blockDim.x) out[b] = R[b];
 }
 
-__global__ void eval_points_kernel(Chain f, int npts, const unsigned char* bits, int max_bond, double* out,
-                                   double* work) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= npts) return;
-  double* v = work + (size_t)warp * 2 * max_bond;
-  const unsigned char* b = bits + (size_t)warp * f.n;
-  const double val = eval_point_warp(f, [b](int n) { return b[n] != 0; }, v, v + max_bond);
-  if (lane == 0) out[warp] = val;
+template <int PT>
+__global__ void __launch_bounds__(kEvalThreads) eval_points_kernel(Chain f, int npts, const unsigned char* bits,
+                                                                   int max_bond, double* out) {
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  const int p0 = blockIdx.x * PT;
+  const unsigned char* b = bits + (size_t)p0 * f.n;
+  const int N = f.n;
+  eval_points_block<PT>(f, [b, N](int p, int n) { return b[(size_t)p * N + n] != 0; }, min(PT, npts - p0), max_bond,
+                        (double*)dyn_smem, out + p0);
 }
 
 __global__ void kron_diag_kernel(Chain om, Chain f, Chain out, const double* hf, int kphi) {
@@ -427,15 +436,27 @@ void left_weight_envs(cudaStream_t st, const Chain& f, const Chain* wchains_dev,
 }
 void right_ones_env(cudaStream_t st, const Chain& f, int n0, int max_bond, double* out, double* work) {
   count_launches(1);
-  right_ones_env_kernel<<<1, 256, 0, st>>>(f, n0, max_bond, out, work);
+  right_ones_env_kernel<<<1, 1024, 0, st>>>(f, n0, max_bond, out, work);
 }
-void eval_points(cudaStream_t st, const Chain& f, int npts, const unsigned char* bits, int max_bond, double* out,
-                 double* work) {
-  if (npts <= 0) return;
-  const int warps_per_block = 8;
+void eval_points(cudaStream_t st, const Chain& f, int npts, const unsigned char* bits, int max_bond, double* out) {
+  const int pt = eval_points_per_block(npts, max_bond);
+  const size_t smem = eval_points_smem(pt, max_bond);
+  static const bool attr = [] {
+    cudaFuncSetAttribute(eval_points_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    cudaFuncSetAttribute(eval_points_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    cudaFuncSetAttribute(eval_points_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    cudaFuncSetAttribute(eval_points_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    return true;
+  }();
+  (void)attr;
+  const unsigned blocks = (unsigned)((npts + pt - 1) / pt);
   count_launches(1);
-  eval_points_kernel<<<(npts + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0, st>>>(
-      f, npts, bits, max_bond, out, work);
+  switch (pt) {
+    case 8: eval_points_kernel<8><<<blocks, kEvalThreads, smem, st>>>(f, npts, bits, max_bond, out); break;
+    case 4: eval_points_kernel<4><<<blocks, kEvalThreads, smem, st>>>(f, npts, bits, max_bond, out); break;
+    case 2: eval_points_kernel<2><<<blocks, kEvalThreads, smem, st>>>(f, npts, bits, max_bond, out); break;
+    default: eval_points_kernel<1><<<blocks, kEvalThreads, smem, st>>>(f, npts, bits, max_bond, out); break;
+  }
 }
 void kron_diag_cores(cudaStream_t st, const Chain& om, const Chain& f, const Chain& out, const double* hf, int kphi) {
   long long most = 1;

@@ -6,9 +6,8 @@
 // reserved by their own pool (a framework's caching allocator that holds the
 // whole GPU), and monitoring loops that probe the PDF every step and must not
 // pay the implicit device-wide synchronisation of cudaFree.
-// qtt_observe_points_noalloc serves them: the query flags, the per-point
-// scratch vectors and the results live in one file-scope device array of
-// fixed size, so the call performs no cudaMalloc, cudaFree or other
+// qtt_observe_points_noalloc serves them: the query flags and the results
+// live in one file-scope device array of fixed size, so the call performs no cudaMalloc, cudaFree or other
 // allocating routine.  It still copies the query in and the values out on the
 // context's stream and synchronises that stream before it returns.
 //
@@ -65,16 +64,27 @@ void* scratch_address(int device) {
 }
 
 // The point-evaluation kernel reading the index bits as the caller's 0/1
-// doubles (the same warp routine as the allocating path, which reads bytes).
-// One warp per point; its two scratch rows sit in the shared array.
-__global__ void eval_points_flags_kernel(Chain f, int npts, const double* flags, int max_bond, double* out,
-                                         double* work) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= npts) return;
-  double* v = work + (size_t)warp * 2 * max_bond;
-  const double* fl = flags + (size_t)warp * f.n;
-  const double val = eval_point_warp(f, [fl](int n) { return fl[n] != 0.0; }, v, v + max_bond);
-  if (lane == 0) out[warp] = val;
+// doubles (the same block routine as the allocating path, which reads bytes).
+template <int PT>
+__global__ void __launch_bounds__(kEvalThreads) eval_points_flags_kernel(Chain f, int npts, const double* flags,
+                                                                         int max_bond, double* out) {
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  const int p0 = blockIdx.x * PT;
+  const double* fl = flags + (size_t)p0 * f.n;
+  const int N = f.n;
+  eval_points_block<PT>(f, [fl, N](int p, int n) { return fl[(size_t)p * N + n] != 0.0; }, min(PT, npts - p0), max_bond,
+                        (double*)dyn_smem, out + p0);
+}
+
+template <int PT>
+void launch_flags(cudaStream_t st, const Chain& f, int npts, const double* flags, int max_bond, double* out) {
+  static const bool attr = [] {
+    cudaFuncSetAttribute(eval_points_flags_kernel<PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    return true;
+  }();
+  (void)attr;
+  eval_points_flags_kernel<PT><<<(npts + PT - 1) / PT, kEvalThreads, eval_points_smem(PT, max_bond), st>>>(
+      f, npts, flags, max_bond, out);
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -82,8 +92,9 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 }  // namespace
 
 size_t Engine::points_noalloc_capacity() const {
-  // per point: its value, its N flags and two scratch rows of the largest
-  // bond of the context; three 256-byte alignment paddings are reserved
+  // the documented limit: per point its value, its N flags and room for two
+  // rows of the largest bond of the context (the rows are in shared memory
+  // now); three 256-byte alignment paddings are reserved
   const size_t per = 8 + 8 * (size_t)N_ + 16 * (size_t)max_bond_;
   const size_t usable = kPointsScratchBytes - 3 * 256;
   return usable / per;
@@ -105,13 +116,15 @@ void Engine::points_noalloc(double* inout, int npts) {
   unsigned char* base = (unsigned char*)scratch_address(device);
   double* vals = (double*)base;
   double* flags = (double*)(base + align256((size_t)npts * 8));
-  double* work = (double*)((unsigned char*)flags + align256((size_t)npts * N_ * 8));
   if (cudaMemcpyAsync(flags, inout, (size_t)npts * N_ * sizeof(double), cudaMemcpyHostToDevice, st_) != cudaSuccess)
     throw std::runtime_error("CUDA error: copy of the point query failed");
-  const int warps_per_block = 8;
   count_launches(1);
-  eval_points_flags_kernel<<<(npts + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0, st_>>>(
-      f_.chain(), npts, flags, max_bond_, vals, work);
+  switch (eval_points_per_block(npts, max_bond_)) {
+    case 8: launch_flags<8>(st_, f_.chain(), npts, flags, max_bond_, vals); break;
+    case 4: launch_flags<4>(st_, f_.chain(), npts, flags, max_bond_, vals); break;
+    case 2: launch_flags<2>(st_, f_.chain(), npts, flags, max_bond_, vals); break;
+    default: launch_flags<1>(st_, f_.chain(), npts, flags, max_bond_, vals); break;
+  }
   if (cudaGetLastError() != cudaSuccess) throw std::runtime_error("CUDA error: point evaluation launch failed");
   if (cudaMemcpyAsync(inout, vals, (size_t)npts * sizeof(double), cudaMemcpyDeviceToHost, st_) != cudaSuccess)
     throw std::runtime_error("CUDA error: copy of the point values failed");

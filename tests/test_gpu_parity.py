@@ -362,3 +362,19 @@ def test_error_measures_match_oracle(sgs):
         assert ref[k] > 1e-4, k
         assert abs(got[k] - ref[k]) <= 1e-9 * ref[k], k
     assert got["err_2c_down"] <= 1e-12 and ref["err_2c_down"] <= 1e-12  # <1> stays 1 point-wise
+
+
+@pytest.mark.parametrize("npts", [1, 3, 5, 250, 2433, 2440])
+def test_point_blocks_match_dense(npts):
+    """Four points to a block up to 2432 points and eight beyond, with partial
+    last blocks; an odd chi above and below one warp of columns (bonds 1 .. 45)."""
+    p = workload.make_params({"bits": 4, "chi_max": 45, "steps": 1})
+    p["bits"] = [2, 3, 3, 4, 3]
+    rng = np.random.default_rng(npts)
+    idx = np.stack([rng.integers(0, 2 ** b, npts) for b in p["bits"]], axis=1)
+    with pkg.qtt_init(p) as ctx:
+        ctx.step(1)
+        dense = ctx.observe(pkg.OBS_DENSE).reshape([2 ** b for b in p["bits"]])
+        vals = ctx.points(idx)
+    # 15 sites of at most 45 terms each in another order: far below 1e-13 of the largest value
+    assert np.abs(vals - dense[tuple(idx.T)]).max() <= 1e-13 * np.abs(dense).max()
