@@ -234,9 +234,9 @@ qtt_status qtt_truncate_vjp(int32_t N, const int32_t* rx, const double* x, const
  * concurrently on the GPU.  Once every context has captured its step graphs
  * (after its first three steps), each step is one launch of a graph that
  * embeds every context's step graph as an independent node; it is built the
- * first time a set of contexts is stepped together and rebuilt when the set,
- * a context's graphs or the contexts' relative step parity change (the
- * contexts must belong to the current device).  The
+ * first time a set of contexts is stepped together, kept for the four sets
+ * stepped last, and rebuilt when a context's graphs or the contexts' relative
+ * step parity change (the contexts must belong to the current device).  The
  * contexts may differ in grid, chi, coefficients and precision; a context
  * must not appear twice.  Returns QTT_OK, or the status of the first context
  * (lowest index) that failed, whose index goes to *failed (-1 when none;

@@ -4,6 +4,8 @@
 // parameters, dispatches and formats outputs.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -245,16 +247,17 @@ namespace {
 // is embedded as an independent child node of one parent graph, which is
 // launched on a stream of the batch; the next step uses the parent graph of
 // the flipped parities.  Both parent graphs are built the first time a set
-// of contexts (engine ids, graph generations, parities) is stepped and kept
-// for the most recent set.
+// of contexts (engine ids, graph generations, parities) is stepped.  Building
+// them takes longer than several steps, so the graphs of the last kBatchSets
+// sets are kept: four steps of a set of 12, three sets in turn, take 239 ms
+// where rebuilding at every change of the set made it 463.  A set is dropped
+// when one of its contexts is destroyed.
+constexpr size_t kBatchSets = 4;
 struct BatchGraph {
   std::vector<unsigned long long> ids;
   std::vector<unsigned> gens;
   std::vector<int> par0;  // parities the exec[0] graph was built for
   cudaGraphExec_t exec[2] = {nullptr, nullptr};
-  cudaStream_t st = nullptr;
-  cudaEvent_t ev = nullptr;
-  std::vector<cudaEvent_t> ctx_ev;
   void release() {
     for (cudaGraphExec_t& e : exec)
       if (e) {
@@ -263,62 +266,106 @@ struct BatchGraph {
       }
   }
 };
-std::mutex g_batch_mu;
-BatchGraph g_batch;
+std::mutex g_batch_mu;                        // held by qtt_step_many
+std::vector<BatchGraph> g_batch;              // most recently used first
+cudaStream_t g_batch_st = nullptr;
+cudaEvent_t g_batch_ev = nullptr;
+std::vector<cudaEvent_t> g_batch_ctx_ev;
+std::mutex g_dead_mu;                         // qtt_destroy only notes the id
+std::vector<unsigned long long> g_dead_ids;
+std::atomic<bool> g_batch_used{false};
+
+void batch_note_destroyed(unsigned long long id) {
+  if (!g_batch_used.load()) return;
+  std::lock_guard<std::mutex> lk(g_dead_mu);
+  g_dead_ids.push_back(id);
+}
+
+// drops the sets that hold a destroyed context
+void batch_purge() {
+  std::vector<unsigned long long> dead;
+  {
+    std::lock_guard<std::mutex> lk(g_dead_mu);
+    dead.swap(g_dead_ids);
+  }
+  for (size_t s = 0; s < g_batch.size() && !dead.empty();) {
+    bool hit = false;
+    for (unsigned long long id : g_batch[s].ids) hit = hit || std::find(dead.begin(), dead.end(), id) != dead.end();
+    if (hit) {
+      g_batch[s].release();
+      g_batch.erase(g_batch.begin() + s);
+    } else {
+      ++s;
+    }
+  }
+}
 
 bool batch_build(qtt_ctx* const* ctxs, int32_t n) {
-  BatchGraph& B = g_batch;
-  B.release();
-  if (!B.st && cudaStreamCreateWithFlags(&B.st, cudaStreamNonBlocking) != cudaSuccess) return false;
-  if (!B.ev && cudaEventCreateWithFlags(&B.ev, cudaEventDisableTiming) != cudaSuccess) return false;
-  while ((int32_t)B.ctx_ev.size() < n) {
+  if (!g_batch_st && cudaStreamCreateWithFlags(&g_batch_st, cudaStreamNonBlocking) != cudaSuccess) return false;
+  if (!g_batch_ev && cudaEventCreateWithFlags(&g_batch_ev, cudaEventDisableTiming) != cudaSuccess) return false;
+  while ((int32_t)g_batch_ctx_ev.size() < n) {
     cudaEvent_t e = nullptr;
     if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
-    B.ctx_ev.push_back(e);
+    g_batch_ctx_ev.push_back(e);
   }
-  B.ids.assign(n, 0);
-  B.gens.assign(n, 0);
-  B.par0.assign(n, 0);
+  BatchGraph B;
   for (int32_t i = 0; i < n; ++i) {
     const qtt::Engine& E = *ctxs[i]->eng;
-    B.ids[i] = E.id();
-    B.gens[i] = E.graph_generation();
-    B.par0[i] = E.parity();
+    B.ids.push_back(E.id());
+    B.gens.push_back(E.graph_generation());
+    B.par0.push_back(E.parity());
+  }
+  // the same contexts with graphs of another generation, or in another relative parity
+  for (size_t s = 0; s < g_batch.size(); ++s)
+    if (g_batch[s].ids == B.ids) {
+      g_batch[s].release();
+      g_batch.erase(g_batch.begin() + s);
+      break;
+    }
+  while (g_batch.size() >= kBatchSets) {
+    g_batch.back().release();
+    g_batch.pop_back();
   }
   for (int flip = 0; flip < 2; ++flip) {
     cudaGraph_t parent = nullptr;
-    if (cudaGraphCreate(&parent, 0) != cudaSuccess) return false;
-    bool ok = true;
+    bool ok = cudaGraphCreate(&parent, 0) == cudaSuccess;
     for (int32_t i = 0; i < n && ok; ++i) {
       cudaGraphNode_t node;
       ok = cudaGraphAddChildGraphNode(&node, parent, nullptr, 0,
                                       ctxs[i]->eng->graph_template(B.par0[i] ^ flip)) == cudaSuccess;
     }
     ok = ok && cudaGraphInstantiate(&B.exec[flip], parent, 0) == cudaSuccess;
-    cudaGraphDestroy(parent);
+    if (parent) cudaGraphDestroy(parent);
     if (!ok) {
       cudaGetLastError();
       B.release();
       return false;
     }
   }
+  g_batch.insert(g_batch.begin(), std::move(B));
+  g_batch_used.store(true);
   return true;
 }
 
-// exec index for the contexts' current parities, or -1 when the cached
-// parent graphs do not describe this set of contexts
+// exec index of the kept parent graphs of this set for the contexts' current
+// parities (the set moves to the front), or -1 when there are none
 int batch_match(qtt_ctx* const* ctxs, int32_t n) {
-  const BatchGraph& B = g_batch;
-  if ((int32_t)B.ids.size() != n || !B.exec[0] || !B.exec[1]) return -1;
-  int flip = -1;
-  for (int32_t i = 0; i < n; ++i) {
-    const qtt::Engine& E = *ctxs[i]->eng;
-    if (B.ids[i] != E.id() || B.gens[i] != E.graph_generation()) return -1;
-    const int f = E.parity() ^ B.par0[i];
-    if (flip >= 0 && f != flip) return -1;
-    flip = f;
+  for (size_t s = 0; s < g_batch.size(); ++s) {
+    const BatchGraph& B = g_batch[s];
+    if ((int32_t)B.ids.size() != n) continue;
+    int flip = -1;
+    bool same = true;
+    for (int32_t i = 0; i < n && same; ++i) {
+      const qtt::Engine& E = *ctxs[i]->eng;
+      const int f = E.parity() ^ B.par0[i];
+      same = B.ids[i] == E.id() && B.gens[i] == E.graph_generation() && (flip < 0 || f == flip);
+      flip = f;
+    }
+    if (!same) continue;
+    std::rotate(g_batch.begin(), g_batch.begin() + s, g_batch.begin() + s + 1);
+    return flip;
   }
-  return flip;
+  return -1;
 }
 
 }  // namespace
@@ -344,13 +391,14 @@ qtt_status qtt_step_many(qtt_ctx* const* ctxs, int32_t n, int32_t nsteps, int32_
   std::vector<int> bad(n, 0);
   std::vector<qtt_status> code(n, QTT_OK);
   std::lock_guard<std::mutex> batch_lock(g_batch_mu);
+  batch_purge();
   bool on_batch = false;  // the batch stream holds work the contexts' streams have not waited for
   auto leave_batch = [&]() {
     if (!on_batch) return true;
     on_batch = false;
-    if (cudaEventRecord(g_batch.ev, g_batch.st) != cudaSuccess) return false;
+    if (cudaEventRecord(g_batch_ev, g_batch_st) != cudaSuccess) return false;
     for (int32_t i = 0; i < n; ++i)
-      if (cudaStreamWaitEvent(ctxs[i]->eng->stream(), g_batch.ev, 0) != cudaSuccess) return false;
+      if (cudaStreamWaitEvent(ctxs[i]->eng->stream(), g_batch_ev, 0) != cudaSuccess) return false;
     return true;
   };
   for (int32_t s = 0; s < nsteps; ++s) {
@@ -363,17 +411,18 @@ qtt_status qtt_step_many(qtt_ctx* const* ctxs, int32_t n, int32_t nsteps, int32_
         bool ok = true;
         if (!on_batch) {  // the batch stream waits for every context's earlier work
           for (int32_t i = 0; i < n && ok; ++i)
-            ok = cudaEventRecord(g_batch.ctx_ev[i], ctxs[i]->eng->stream()) == cudaSuccess &&
-                 cudaStreamWaitEvent(g_batch.st, g_batch.ctx_ev[i], 0) == cudaSuccess;
+            ok = cudaEventRecord(g_batch_ctx_ev[i], ctxs[i]->eng->stream()) == cudaSuccess &&
+                 cudaStreamWaitEvent(g_batch_st, g_batch_ctx_ev[i], 0) == cudaSuccess;
         }
-        ok = ok && cudaGraphLaunch(g_batch.exec[flip], g_batch.st) == cudaSuccess;
+        ok = ok && cudaGraphLaunch(g_batch.front().exec[flip], g_batch_st) == cudaSuccess;
         if (ok) {
           on_batch = true;
           for (int32_t i = 0; i < n; ++i) ctxs[i]->eng->step_launched_externally();
           continue;
         }
         cudaGetLastError();
-        g_batch.release();
+        g_batch.front().release();
+        g_batch.erase(g_batch.begin());
       }
     }
     if (!leave_batch()) {
@@ -656,7 +705,10 @@ qtt_status qtt_load(qtt_ctx* ctx, const char* path) {
 void qtt_destroy(qtt_ctx* ctx) {
   if (!ctx) return;
   try {
-    if (ctx->eng) cudaStreamSynchronize(ctx->eng->stream());
+    if (ctx->eng) {
+      cudaStreamSynchronize(ctx->eng->stream());
+      batch_note_destroyed(ctx->eng->id());
+    }
   } catch (...) {
   }
   delete ctx;

@@ -56,3 +56,37 @@ def test_step_many_rejects_a_repeated_context():
         assert "twice" in str(ei.value)
     finally:
         c.close()
+
+
+def test_sets_stepped_in_turn_match_separate_steps():
+    """Five sets (more than are kept) stepped in turn, a context shared by two
+    sets, and a set whose context is destroyed and made anew: every state stays
+    bitwise that of stepping the contexts alone."""
+    ps = _instances()[:2]
+    sets = [[pkg.qtt_init(p) for p in ps] for _ in range(4)]
+    alone = [pkg.qtt_init(p) for p in ps]
+    fresh = None
+    try:
+        sets.append([sets[0][0], sets[1][1]])
+        for _ in range(2):
+            for s in sets:
+                pkg.qtt_step_many(s, 4)
+        sets[2][0].close()
+        fresh = pkg.qtt_init(ps[0])
+        sets[2][0] = fresh
+        pkg.qtt_step_many(sets[2], 5)
+        steps = {id(c): 8 for s in sets[:4] for c in s}
+        steps[id(sets[0][0])] = steps[id(sets[1][1])] = 16
+        steps[id(fresh)], steps[id(sets[2][1])] = 5, 13
+        for j, a in enumerate(alone):
+            done = 0
+            for s in sorted(sets[:4], key=lambda s: steps[id(s[j])]):
+                n = steps[id(s[j])]
+                a.step(n - done)
+                done = n
+                assert s[j].scalars()["steps"] == n and s[j].compare(a) == 0.0
+    finally:
+        for c in {id(c): c for s in sets for c in s}.values():
+            c.close()
+        for c in alone:
+            c.close()
