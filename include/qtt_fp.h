@@ -352,7 +352,11 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *      kind (0 FP64, 1 small products in FP64, 2 in FP32), the terms of a dot
  *      product and max |C - C_host| / (|alpha| sum |a b| + |beta c0|)
  *   8  FP64 eigensolver on a batch of 14 problems of different sizes, the
- *      leading k columns: the three values of 2 per problem */
+ *      leading k columns: the three values of 2 per problem
+ *   9  one-launch tensor-core GEMM (TF32X3, BF16X6, BF16X10) on seeded
+ *      operands against a host sum: per case the mode's enum value, the terms
+ *      of a dot product, max and mean of (C - C_host) / (|alpha| sum |a b| +
+ *      |beta c0|), or -1, 0 where it does not take the shape */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

@@ -84,6 +84,8 @@ struct KernelTimer {
 };
 enum { TM_GEMM = 0, TM_QR = 1, TM_EIG = 2, TM_OTHER = 3, TM_TC = 4, TM_SMALL = 5 };
 
+constexpr double kTcPasses[6] = {3, 2, 6, 1, 6, 10};  // MMA passes by TcMode, in bf16-pass units
+
 struct TimeScope {
   KernelTimer* t;
   int cls;
@@ -99,6 +101,14 @@ struct TimeScope {
   }
   ~TimeScope() {
     if (t && t->on && b) cudaEventRecord(b, st);
+  }
+  void drop() {  // nothing was launched: forget the record
+    if (t && t->on && b) {
+      t->pool.push_back(t->recs.back().a);
+      t->pool.push_back(b);
+      t->recs.pop_back();
+      b = nullptr;
+    }
   }
 };
 
@@ -270,6 +280,20 @@ bool Engine::small_in_fp32(int role) const {
   return tc_mode_[role] >= 0 && (small_fp32_ || (small_sketch_fp32_ && role != GEMM_STATE && role != GEMM_MIX));
 }
 
+bool Engine::gemm_one_launch(int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B, double beta,
+                             OutView C, const SumPieces& P, int role) {
+  const int mode = tc_mode_[role];
+  if (mode < 0) return false;
+  const double fl = 2.0 * M * (double)N * K * outer * inner * P.n;
+  TimeScope ts(timer_, TM_TC, cur(), fl);
+  if (!gemm_fused(cur(), mode, M, N, K, outer, inner, alpha, A, B, beta, C, P, lane_ws_[lane_], ws_elems_, status_ + 2)) {
+    ts.drop();
+    return false;
+  }
+  if (timer_->on) tc_issued_flops_ += fl * kTcPasses[mode];
+  return true;
+}
+
 void Engine::gemm_sum(int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B, OutView C,
                       const SumPieces& P, int role) {
   if (small_gemm_fits(M, N, K, outer, inner)) {
@@ -277,6 +301,7 @@ void Engine::gemm_sum(int M, int N, int K, int outer, int inner, double alpha, M
     small_gemm_sum(cur(), small_in_fp32(role), M, N, K, outer, inner, alpha, A, B, 0.0, C, P);
     return;
   }
+  if (gemm_one_launch(M, N, K, outer, inner, alpha, A, B, 0.0, C, P, role)) return;
   for (int p = 0; p < P.n; ++p) {
     MatView Ap = A, Bp = B;
     Ap.p += p * P.a;
@@ -298,6 +323,7 @@ void Engine::gemm(int M, int N, int K, int outer, int inner, double alpha, MatVi
     gemm64(M, N, K, outer, inner, alpha, A, B, beta, C);
     return;
   }
+  if (gemm_one_launch(M, N, K, outer, inner, alpha, A, B, beta, C, SumPieces{}, role)) return;
   const size_t need = tc_workspace_bytes(M, N, K, (long long)outer * inner, mode);
   void*& pw = pack_ws_[lane_];
   size_t& pb = pack_bytes_[lane_];
@@ -315,10 +341,7 @@ void Engine::gemm(int M, int N, int K, int outer, int inner, double alpha, MatVi
     pb = bytes;
   }
   const double fl = 2.0 * M * (double)N * K * outer * inner;
-  if (timer_->on) {
-    static const double passes[6] = {3, 2, 6, 1, 6, 10};  // indexed by TcMode, in bf16-pass units
-    tc_issued_flops_ += fl * passes[mode];
-  }
+  if (timer_->on) tc_issued_flops_ += fl * kTcPasses[mode];
   TimeScope ts(timer_, TM_TC, cur(), fl);
   if (!gemm_tc(cur(), mode, M, N, K, outer, inner, alpha, A, B, beta, C, pw, pb, lane_ws_[lane_], ws_elems_,
                status_ + 2))

@@ -184,6 +184,9 @@ class Engine {
   // alpha sum_p A_p B_p over the pieces: one launch where the product is small, else one product per piece
   void gemm_sum(int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B, OutView C,
                 const SumPieces& P, int role);
+  // the tensor-core product without packing passes, where its shape allows; false: nothing launched
+  bool gemm_one_launch(int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B, double beta,
+                       OutView C, const SumPieces& P, int role);
   bool small_in_fp32(int role) const;  // arithmetic of the small products of a role
   // FP64 product (Gram matrices, norms, masses, observables).
   void gemm64(int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B, double beta, OutView C);

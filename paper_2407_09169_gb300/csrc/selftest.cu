@@ -79,6 +79,9 @@ std::vector<double> down(const double* d, size_t n) {
 // which = 8: the FP64 eigensolver on a batch of problems of different sizes:
 // per problem ||G U - U diag(lam)|| / ||G||, ||U^T U - I||_max and 1 if the
 // eigenvalues are not descending, for the leading k columns.
+// which = 9: the one-launch tensor-core GEMM against a host sum: per case the
+// mode, the terms of a dot product, max and mean of (C - C_host) / (|alpha|
+// sum |a b| + |beta c0|); -1 where it does not take the shape.
 std::vector<double> run_selftest(int which) {
   cudaStream_t st = nullptr;
   std::vector<double> out;
@@ -637,6 +640,94 @@ std::vector<double> run_selftest(int which) {
       out.push_back(res / gn);
       out.push_back(orth);
       out.push_back(order);
+    }
+  } else if (which == 9) {
+    struct Case {
+      int mode, M, N, K, outer, inner, pieces;
+      bool ta, tb, sa, sb;  // transposed operands; operands that do not depend on the outer index
+      double alpha, beta;
+      bool flip_c;  // C column-major
+    };
+    const Case cases[] = {
+        // rows and columns inside one tile, over tile edges, ragged K; every layout of the rows
+        {TC_TF32X3, 128, 144, 32, 1, 1, 1, false, false, false, false, 1.0, 0.0, false},
+        {TC_TF32X3, 300, 136, 136, 1, 2, 1, false, true, false, true, 1.0, 0.0, false},
+        {TC_TF32X3, 77, 85, 77, 9, 2, 1, false, false, true, false, 1.0, 0.0, false},
+        {TC_TF32X3, 128, 136, 77, 5, 1, 2, false, false, true, false, 1.0, 0.0, false},
+        {TC_TF32X3, 272, 136, 3000, 1, 1, 1, false, false, false, false, 1.0, 0.0, false},
+        {TC_TF32X3, 1, 33, 65, 1, 1, 1, true, true, false, false, -1.0, 0.5, true},
+        {TC_BF16X6, 136, 700, 272, 1, 1, 1, true, false, false, false, 1.0, 0.0, false},
+        {TC_BF16X6, 650, 256, 128, 1, 1, 1, false, false, false, false, 0.5, 0.0, false},
+        {TC_BF16X6, 77, 77, 77, 12, 2, 1, true, false, true, false, 1.0, 0.0, false},
+        {TC_BF16X6, 45, 37, 340, 3, 1, 1, false, true, false, true, 1.0, 1.0, true},
+        {TC_BF16X10, 136, 300, 272, 1, 1, 1, true, false, false, false, 1.0, 0.0, false},
+        {TC_BF16X10, 400, 256, 77, 1, 1, 1, false, false, false, false, -1.0, 0.0, false},
+        {TC_BF16X10, 33, 40, 65, 7, 2, 1, false, false, true, false, 1.5, 1.0, false},
+        {TC_BF16X10, 130, 16, 9, 1, 3, 1, true, true, false, false, 1.0, 0.0, true},
+        {TC_BF16X10, 400, 500, 64, 1, 1, 1, false, false, false, false, 1.0, 0.0, false}};
+    const size_t ws_elems = (size_t)8 << 20;
+    DBuf ws(ws_elems);
+    unsigned long long seed = 99;
+    for (const Case& c : cases) {
+      const long long batch = (long long)c.outer * c.inner;
+      const size_t am = (size_t)c.M * c.K, bm = (size_t)c.K * c.N, cm = (size_t)c.M * c.N;
+      const long long na = (c.sa ? c.inner : batch) * c.pieces, nb = (c.sb ? c.inner : batch) * c.pieces;
+      DBuf A(am * na), B(bm * nb), C0(cm * batch);
+      fill_gaussian(st, A.p, am * na, 1.0, seed++, 1);
+      fill_gaussian(st, B.p, bm * nb, 1.0, seed++, 2);
+      fill_gaussian(st, C0.p, cm * batch, 1.0, seed++, 3);
+      const std::vector<double> ha = down(A.p, am * na), hb = down(B.p, bm * nb), hc = down(C0.p, cm * batch);
+      MatView av, bv;
+      OutView cv;
+      av.p = A.p;
+      av.rs = c.ta ? 1 : c.K;
+      av.cs = c.ta ? c.M : 1;
+      av.si = (long long)am * c.pieces;
+      av.so = c.sa ? 0 : av.si * c.inner;
+      bv.p = B.p;
+      bv.rs = c.tb ? 1 : c.N;
+      bv.cs = c.tb ? c.K : 1;
+      bv.si = (long long)bm * c.pieces;
+      bv.so = c.sb ? 0 : bv.si * c.inner;
+      cv.p = C0.p;
+      cv.rs = c.flip_c ? 1 : c.N;
+      cv.cs = c.flip_c ? c.M : 1;
+      cv.si = (long long)cm;
+      cv.so = cv.si * c.inner;
+      SumPieces P;
+      P.n = c.pieces;
+      P.a = (long long)am;
+      P.b0 = (long long)bm;
+      out.push_back((double)c.mode);
+      out.push_back((double)c.K * c.pieces);
+      if (!gemm_fused(st, c.mode, c.M, c.N, c.K, c.outer, c.inner, c.alpha, av, bv, c.beta, cv, P, ws.p, ws_elems, err)) {
+        out.push_back(-1.0);
+        out.push_back(0.0);
+        continue;
+      }
+      const std::vector<double> got = down(C0.p, cm * batch);
+      double worst = 0.0, mean = 0.0;
+      for (long long b = 0; b < batch; ++b)
+        for (int m = 0; m < c.M; ++m)
+          for (int n = 0; n < c.N; ++n) {
+            double v = 0.0, mag = 0.0;
+            for (int p = 0; p < c.pieces; ++p) {
+              const double* a = ha.data() + ((c.sa ? b % c.inner : b) * c.pieces + p) * am;
+              const double* w = hb.data() + ((c.sb ? b % c.inner : b) * c.pieces + p) * bm;
+              for (int k = 0; k < c.K; ++k) {
+                const double t = a[c.ta ? (size_t)k * c.M + m : (size_t)m * c.K + k] *
+                                 w[c.tb ? (size_t)n * c.K + k : (size_t)k * c.N + n];
+                v += t;
+                mag += std::fabs(t);
+              }
+            }
+            const size_t e = (size_t)b * cm + (c.flip_c ? (size_t)n * c.M + m : (size_t)m * c.N + n);
+            const double d = (got[e] - c.alpha * v - c.beta * hc[e]) / (std::fabs(c.alpha) * mag + std::fabs(c.beta * hc[e]));
+            worst = std::fabs(d) > worst || std::isnan(d) ? std::fabs(d) : worst;
+            mean += d / ((double)cm * batch);
+          }
+      out.push_back(worst);
+      out.push_back(mean);
     }
   } else {
     cudaFree(err);

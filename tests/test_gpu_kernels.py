@@ -170,3 +170,22 @@ def test_batched_eigensolver_of_mixed_sizes():
     v = np.array(pkg.qtt_selftest(8)[:-1]).reshape(-1, 3)
     assert v.shape[0] == 14
     assert (v[:, :2] < 1e-12).all() and (v[:, 2] == 0).all(), v
+
+
+def test_one_launch_tensor_core_gemm():
+    """Tile edges, ragged K, both operand layouts, flat rows over the outer
+    batch on either side, two pieces, a K split over CTAs, two chunks of K in
+    BF16X10, alpha and beta, a column-major C; the last shape is too wide and
+    must be refused.  Bounds as for the packed GEMM (see
+    test_tensor_core_gemm_against_host_fp64); the exact-slice forms keep their
+    signed mean far below their bound."""
+    v = np.array(pkg.qtt_selftest(9))
+    assert v[-1] == 0, "a bounded wait gave up"
+    v = v[:-1].reshape(-1, 4)
+    assert v.shape[0] == 15 and v[-1, 2] == -1
+    for mode, terms, worst, mean in v[:-1]:
+        m = MODES[int(mode)]
+        bound = {"tf32x3": 3 * 2.0 ** -22 + (terms / 8) * 2.0 ** -23, "bf16x6": 4.5e-6, "bf16x10": 4.5e-6 * 2.0 ** -7}[m]
+        assert 0 <= worst <= bound, (m, terms, worst)
+        if m != "tf32x3":
+            assert abs(mean) <= 0.05 * bound, (m, terms, mean)
