@@ -356,7 +356,10 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *   9  one-launch tensor-core GEMM (TF32X3, BF16X6, BF16X10) on seeded
  *      operands against a host sum: per case the mode's enum value, the terms
  *      of a dot product, max and mean of (C - C_host) / (|alpha| sum |a b| +
- *      |beta c0|), or -1, 0 where it does not take the shape */
+ *      |beta c0|), or -1, 0 where it does not take the shape
+ *  10  Householder QR at the edges of the kernels' sizes, each on a Gaussian
+ *      matrix, one with zero and repeated columns and one with graded columns
+ *      and rows: as 1, with the residual of the worst column */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

@@ -3,6 +3,7 @@
 #include <cmath>
 #include <stdexcept>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "gemm_tc.cuh"
@@ -151,48 +152,73 @@ std::vector<double> run_selftest(int which) {
       }
     }
     cudaFree(pack);
-  } else if (which == 1) {
-    const int shapes[][2] = {{272, 136}, {64, 33}, {256, 256}, {40, 1}, {288, 143}, {150, 77}, {200, 120}, {96, 2},
-                             {288, 144}, {160, 80}, {97, 49}, {161, 81}, {144, 72}};
-    for (auto& sh : shapes) {
-      const int m = sh[0], n = sh[1];
-      DBuf Y((size_t)m * n), Q((size_t)m * n), W((size_t)2 * m * n + n + 64), Qf((size_t)m * n),
-          G((size_t)8 * n * n);
-      fill_gaussian(st, Y.p, (size_t)m * n, 1.0, 99 + m, 5);
-      // FP64 QR; float QR; float QR + one FP64 Newton-Schulz step
-      for (int run = 0; run < 3; ++run) {
-        if (run < 2) {
-          qr_thin(st, m, n, Y.p, Q.p, W.p, run == 0 ? 64 : 32, err);
-        } else {
-          qr_thin(st, m, n, Y.p, Qf.p, W.p, 32, err);
-          newton_schulz_step(st, m, n, Qf.p, G.p, Q.p);
-        }
+  } else if (which == 1 || which == 10) {
+    // which = 1: Gaussian Y.  which = 10, at the edges of the kernels' sizes: kind 0 Gaussian, 1 every
+    // third column zero and a repeated one, 2 columns scaled by 10^(-12 .. 12) and rows by 1 or 10^-9
+    // (the residual of the worst column).
+    const std::vector<std::pair<int, int>> shapes =
+        which == 1 ? std::vector<std::pair<int, int>>{{272, 136}, {64, 33}, {256, 256}, {40, 1}, {288, 143},
+                                                      {150, 77}, {200, 120}, {96, 2}, {288, 144}, {160, 80},
+                                                      {97, 49}, {161, 81}, {144, 72}}
+                   : std::vector<std::pair<int, int>>{{1, 1},    {3, 2},    {32, 32},   {33, 17},  {96, 48},
+                                                      {49, 49},  {81, 81},  {224, 112}, {225, 112}, {113, 113},
+                                                      {129, 65}, {385, 24}, {384, 100}};
+    for (auto& sh : shapes)
+      for (int kind = 0; kind < (which == 1 ? 1 : 3); ++kind) {
+        const int m = sh.first, n = sh.second;
+        DBuf Y((size_t)m * n), Q((size_t)m * n), W((size_t)2 * m * n + n + 64), Qf((size_t)m * n),
+            G((size_t)8 * n * n);
+        fill_gaussian(st, Y.p, (size_t)m * n, 1.0, 99 + m, 5);
         if (cudaStreamSynchronize(st) != cudaSuccess) throw std::runtime_error("CUDA error: selftest qr");
-        std::vector<double> y = down(Y.p, (size_t)m * n), q = down(Q.p, (size_t)m * n);
-        double orth = 0;
-        for (int a = 0; a < n; ++a)
-          for (int b2 = 0; b2 < n; ++b2) {
-            double s = 0;
-            for (int i = 0; i < m; ++i) s += q[(size_t)i * n + a] * q[(size_t)i * n + b2];
-            orth = std::fmax(orth, std::fabs(s - (a == b2 ? 1.0 : 0.0)));
-          }
-        // projection residual ||Y - Q Q^T Y||_F / ||Y||_F
-        double num = 0, den = 0;
-        for (int c = 0; c < n; ++c) {
-          std::vector<double> coef(n, 0.0);
-          for (int a = 0; a < n; ++a)
-            for (int i = 0; i < m; ++i) coef[a] += q[(size_t)i * n + a] * y[(size_t)i * n + c];
-          for (int i = 0; i < m; ++i) {
-            double r = y[(size_t)i * n + c];
-            for (int a = 0; a < n; ++a) r -= q[(size_t)i * n + a] * coef[a];
-            num += r * r;
-            den += y[(size_t)i * n + c] * y[(size_t)i * n + c];
-          }
+        std::vector<double> y = down(Y.p, (size_t)m * n);
+        if (kind > 0) {
+          for (int i = 0; i < m; ++i)
+            for (int c = 0; c < n; ++c) {
+              double& v = y[(size_t)i * n + c];
+              if (kind == 1) v = c % 3 == 2 ? 0.0 : c > 0 && c % 3 == 0 ? y[(size_t)i * n + c - 2] : v;
+              if (kind == 2) v *= std::pow(10.0, 12 * (c % 3 - 1)) * ((i + c) % 3 == 0 ? 1e-9 : 1.0);
+            }
+          if (cudaMemcpy(Y.p, y.data(), y.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+            throw std::runtime_error("CUDA error: selftest qr");
         }
-        out.push_back(orth);
-        out.push_back(std::sqrt(num / den));
+        // FP64 QR; float QR; float QR + one FP64 Newton-Schulz step
+        for (int run = 0; run < 3; ++run) {
+          if (run < 2) {
+            qr_thin(st, m, n, Y.p, Q.p, W.p, run == 0 ? 64 : 32, err);
+          } else {
+            qr_thin(st, m, n, Y.p, Qf.p, W.p, 32, err);
+            newton_schulz_step(st, m, n, Qf.p, G.p, Q.p);
+          }
+          if (cudaStreamSynchronize(st) != cudaSuccess) throw std::runtime_error("CUDA error: selftest qr");
+          std::vector<double> q = down(Q.p, (size_t)m * n);
+          double orth = 0;
+          for (int a = 0; a < n; ++a)
+            for (int b2 = 0; b2 < n; ++b2) {
+              double s = 0;
+              for (int i = 0; i < m; ++i) s += q[(size_t)i * n + a] * q[(size_t)i * n + b2];
+              orth = std::fmax(orth, std::fabs(s - (a == b2 ? 1.0 : 0.0)));
+            }
+          // projection residual ||Y - Q Q^T Y||_F / ||Y||_F, or of the worst column
+          double num = 0, den = 0, worst = 0;
+          for (int c = 0; c < n; ++c) {
+            std::vector<double> coef(n, 0.0);
+            double cn = 0, cd = 0;
+            for (int a = 0; a < n; ++a)
+              for (int i = 0; i < m; ++i) coef[a] += q[(size_t)i * n + a] * y[(size_t)i * n + c];
+            for (int i = 0; i < m; ++i) {
+              double r = y[(size_t)i * n + c];
+              for (int a = 0; a < n; ++a) r -= q[(size_t)i * n + a] * coef[a];
+              cn += r * r;
+              cd += y[(size_t)i * n + c] * y[(size_t)i * n + c];
+            }
+            num += cn;
+            den += cd;
+            if (cd > 0) worst = std::fmax(worst, std::sqrt(cn / cd));
+          }
+          out.push_back(orth);
+          out.push_back(which == 1 ? std::sqrt(num / den) : worst);
+        }
       }
-    }
   } else if (which == 2) {
     // (size, spectrum): 0 G = X diag(10^(-6 k / n)) X^T (X Gaussian); with Q
     // orthonormal (Gram-Schmidt of a Gaussian X on the host) G = Q diag(w) Q^T

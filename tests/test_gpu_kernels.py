@@ -189,3 +189,19 @@ def test_one_launch_tensor_core_gemm():
         assert 0 <= worst <= bound, (m, terms, worst)
         if m != "tf32x3":
             assert abs(mean) <= 0.05 * bound, (m, terms, mean)
+
+
+def test_householder_qr_edges():
+    """Edges of the panels (16 CPW columns, 32 RPL rows), odd rows, square and
+    one-column matrices, one past the largest register variant, rank-deficient
+    and graded columns (1e-12 to 1e12: no sum of squares leaves the float range).
+    Householder QR is backward stable column by column, so the bounds are those
+    of test_householder_qr with the worst column's residual."""
+    v = np.array(pkg.qtt_selftest(10))
+    assert v[-1] == 0, "a bounded wait gave up, or a factor was not finite"
+    v = v[:-1].reshape(-1, 3, 2)
+    assert v.shape[0] == 13 * 3
+    for (o64, r64), (o32, r32), (ons, rns) in v:
+        assert o64 < 1e-13 and r64 < 1e-13
+        assert o32 < 2e-5 and r32 < 2e-5
+        assert ons <= 0.75 * 256 * o32 ** 2 + 2e-12 and rns < 2e-5
