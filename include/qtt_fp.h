@@ -359,7 +359,9 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *      |beta c0|), or -1, 0 where it does not take the shape
  *  10  Householder QR at the edges of the kernels' sizes, each on a Gaussian
  *      matrix, one with zero and repeated columns and one with graded columns
- *      and rows: as 1, with the residual of the worst column */
+ *      and rows: as 1, with the residual of the worst column
+ *  11  FP64 eigensolver on four batches at the edges of the back-transform's
+ *      variants (12 problems): the three values of 2 per problem */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

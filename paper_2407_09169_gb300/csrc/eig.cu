@@ -1225,6 +1225,84 @@ __global__ void __launch_bounds__(32 * BT_WARPS) eig_back_transform(const EigPro
   }
 }
 
+// The same in FP64 for n <= 32 NG, with eight lanes per vector and the vectors in
+// registers: lane q of a vector holds its rows q + 8 t, in groups of four t that
+// a reflector below them skips.  What bounds it is a warp's FP64 instructions, 64
+// clocks each with none overlapping (four warps of an SM do): with the vectors in
+// shared memory the loads of the reflector and of the vector came on top.  The
+// next reflector is loaded meanwhile; with four lanes per vector (half the
+// reduction steps) its 36 loads no longer fit the registers and wait.
+// The whole eigensolver, 25 problems of n = 136 with 128 vectors: 2.71 -> 2.45 ms,
+// 3 of them 2.12 -> 1.83, 17 of n = 72 1.00 -> 0.91.  Larger problems keep the
+// vectors in shared memory (above).
+template <int NG>
+__global__ void __launch_bounds__(64) eig_back_transform_reg(const EigProblem* __restrict__ probs) {
+  constexpr int LPV = 8, VECS = 32 / LPV, NR = 4 * NG;  // lanes per vector, vectors per warp, rows per lane
+  const EigProblem P = probs[blockIdx.y];
+  const int n = P.n, k = P.k;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = (blockIdx.x * 2 + w) * VECS;
+  if (r0 >= k) return;
+  const EigLayout L = eig_layout<double>(n);
+  const double* W = (const double*)P.work;
+  const int* I = (const int*)(P.work + L.ints_off);
+  const double* A = W + L.A;
+  const double* Z = W + ((dc_depth(n) & 1) ? L.dcV : L.Z);
+  const int q = lane % LPV, r = r0 + lane / LPV;
+  const int col = r < k ? I[L.order + r] : 0;
+  double z[NR], an[NR], taun = 0.0;
+#pragma unroll
+  for (int t = 0; t < NR; ++t) {
+    const int x = q + LPV * t;
+    z[t] = (r < k && x < n) ? Z[(size_t)x * n + col] : 0.0;
+  }
+  auto load = [&](int j) {  // v_j: 1 in row j + 1, zeros above
+    taun = A[(size_t)j * n + j];
+#pragma unroll
+    for (int t = 0; t < NR; ++t) {
+      const int x = q + LPV * t;
+      an[t] = (x > j + 1 && x < n) ? A[(size_t)j * n + x] : (x == j + 1 ? 1.0 : 0.0);
+    }
+  };
+  if (n > 2) load(n - 3);
+  for (int j = n - 3; j >= 0; --j) {
+    const double tau = taun;
+    double a[NR];
+#pragma unroll
+    for (int t = 0; t < NR; ++t) a[t] = an[t];
+    if (j > 0) load(j - 1);
+    double d = 0.0;
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+      if (4 * LPV * (g + 1) > j + 1)
+#pragma unroll
+        for (int t = 4 * g; t < 4 * g + 4; ++t) d = fma(a[t], z[t], d);
+#pragma unroll
+    for (int o = 1; o < LPV; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    const double f = -tau * d;
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+      if (4 * LPV * (g + 1) > j + 1)
+#pragma unroll
+        for (int t = 4 * g; t < 4 * g + 4; ++t) z[t] = fma(f, a[t], z[t]);
+  }
+#pragma unroll
+  for (int t = 0; t < NR; ++t) {
+    const int x = q + LPV * t;
+    if (r < k && x < n) P.U[(size_t)x * k + r] = z[t];
+  }
+}
+
+// false where n is too large for the registers
+inline bool back_transform_reg(cudaStream_t st, const EigProblem* probs_dev, int nprob, int nmax, int kmax) {
+  const dim3 grid((kmax + 7) / 8, nprob);
+  if (nmax <= 64) eig_back_transform_reg<2><<<grid, 64, 0, st>>>(probs_dev);
+  else if (nmax <= 96) eig_back_transform_reg<3><<<grid, 64, 0, st>>>(probs_dev);
+  else if (nmax <= 160) eig_back_transform_reg<5><<<grid, 64, 0, st>>>(probs_dev);
+  else return false;
+  return true;
+}
+
 template <typename T>
 void eig_launch(cudaStream_t st, const EigProblem* probs_dev, int nprob, int nmax, int kmax, int* status) {
   const size_t smem_A = (size_t)nmax * (nmax + 1) * sizeof(T);  // row stride n + 1 in shared memory
@@ -1268,6 +1346,9 @@ void eig_launch(cudaStream_t st, const EigProblem* probs_dev, int nprob, int nma
         probs_dev);
   }
   if (kmax > 0) {
+    if constexpr (dc) {
+      if (back_transform_reg(st, probs_dev, nprob, nmax, kmax)) return;
+    }
     const int per_block = BT_WARPS * BT_VECS;
     const size_t bt_smem = (size_t)per_block * nmax * sizeof(T);
     static bool battr = false;

@@ -596,76 +596,80 @@ std::vector<double> run_selftest(int which) {
       out.push_back((double)c.K * c.pieces);
       out.push_back(worst);
     }
-  } else if (which == 8) {
-    // sizes at the edges of the leaves (12) and of the levels; every second
-    // problem of rank n / 3 (equal poles and negligible z in its merges)
-    const int sizes[] = {136, 1, 2, 12, 13, 24, 25, 40, 49, 72, 96, 97, 104, 193};
-    const int np = (int)(sizeof(sizes) / sizeof(sizes[0]));
-    std::vector<std::vector<double>> gs(np);
-    std::vector<EigProblem> probs(np);
-    size_t total = 0;
-    for (int n : sizes) total += 3 * (size_t)n * n + n + eig_work_bytes(n, 64) / 8 + 96;
-    DBuf mem(total), dev(np * sizeof(EigProblem) / 8 + 8);
-    double* p = mem.p;
-    int nmax = 0, kmax = 0;
-    for (int t = 0; t < np; ++t) {
-      const int n = sizes[t];
-      EigProblem& P = probs[t];
-      P.n = n;
-      P.k = t % 3 == 0 ? n : n / 2 + 1;
-      double* X = p;
-      double* G = X + (size_t)n * n;
-      P.G = G;
-      P.U = G + (size_t)n * n;
-      P.lam = P.U + (size_t)n * n;
-      P.work = (unsigned char*)(P.lam + n);
-      P.work = (unsigned char*)(((uintptr_t)P.work + 255) & ~(uintptr_t)255);
-      p = (double*)(((uintptr_t)P.work + eig_work_bytes(n, 64) + 255) & ~(uintptr_t)255);
-      nmax = n > nmax ? n : nmax;
-      kmax = P.k > kmax ? P.k : kmax;
-      fill_gaussian(st, X, (size_t)n * n, 1.0, 555 + t, 6);
-      const std::vector<double> x = down(X, (size_t)n * n);
-      std::vector<double>& g = gs[t];
-      g.assign((size_t)n * n, 0.0);
-      for (int i = 0; i < n; ++i)
-        for (int j = 0; j <= i; ++j) {
-          double s = 0;
-          for (int k = 0; k < n; ++k)
-            s += x[(size_t)i * n + k] * x[(size_t)j * n + k] *
-                 (t % 2 ? (3 * k < n ? 1.0 : 0.0) : std::pow(10.0, -6.0 * k / n));
-          g[(size_t)i * n + j] = g[(size_t)j * n + i] = s;
-        }
-      if (cudaMemcpy(G, g.data(), g.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
-        throw std::runtime_error("CUDA error: selftest eig upload");
-    }
-    if (cudaMemcpy(dev.p, probs.data(), np * sizeof(EigProblem), cudaMemcpyHostToDevice) != cudaSuccess)
-      throw std::runtime_error("CUDA error: selftest eig upload");
-    eig_sym_batched(st, (const EigProblem*)dev.p, np, nmax, kmax, 64, err);
-    if (cudaStreamSynchronize(st) != cudaSuccess) throw std::runtime_error("CUDA error: selftest eig");
-    for (int t = 0; t < np; ++t) {
-      const int n = probs[t].n, k = probs[t].k;
-      const std::vector<double> u = down(probs[t].U, (size_t)n * k), lam = down(probs[t].lam, n);
-      double gn = 0, res = 0, orth = 0, order = 0;
-      for (double v : gs[t]) gn = std::fmax(gn, std::fabs(v));
-      for (int c = 1; c < n; ++c)
-        if (lam[c] > lam[c - 1]) order = 1;
-      for (int c = 0; c < k; ++c) {
-        for (int i = 0; i < n; ++i) {
-          double s = 0;
-          for (int q = 0; q < n; ++q) s += gs[t][(size_t)i * n + q] * u[(size_t)q * k + c];
-          const double d = std::fabs(s - lam[c] * u[(size_t)i * k + c]);
-          res = d > res || std::isnan(d) ? d : res;
-        }
-        for (int c2 = 0; c2 < k; ++c2) {
-          double s = 0;
-          for (int q = 0; q < n; ++q) s += u[(size_t)q * k + c] * u[(size_t)q * k + c2];
-          const double d = std::fabs(s - (c == c2 ? 1.0 : 0.0));
-          orth = d > orth || std::isnan(d) ? d : orth;
-        }
+  } else if (which == 8 || which == 11) {
+    // 8: sizes at the edges of the leaves (12) and of the levels.  11: batches at
+    // the edges of the back-transform's variants.  Every second problem of rank
+    // n / 3 (equal poles and negligible z in its merges).
+    std::vector<std::vector<int>> batches = {{136, 1, 2, 12, 13, 24, 25, 40, 49, 72, 96, 97, 104, 193}};
+    if (which == 11) batches = {{64, 33, 3}, {96, 65, 2, 1}, {160, 97, 145}, {161, 5}};
+    for (const std::vector<int>& sizes : batches) {
+      const int np = (int)sizes.size();
+      std::vector<std::vector<double>> gs(np);
+      std::vector<EigProblem> probs(np);
+      size_t total = 0;
+      for (int n : sizes) total += 3 * (size_t)n * n + n + eig_work_bytes(n, 64) / 8 + 96;
+      DBuf mem(total), dev(np * sizeof(EigProblem) / 8 + 8);
+      double* p = mem.p;
+      int nmax = 0, kmax = 0;
+      for (int t = 0; t < np; ++t) {
+        const int n = sizes[t];
+        EigProblem& P = probs[t];
+        P.n = n;
+        P.k = t % 3 == 0 ? n : n / 2 + 1;
+        double* X = p;
+        double* G = X + (size_t)n * n;
+        P.G = G;
+        P.U = G + (size_t)n * n;
+        P.lam = P.U + (size_t)n * n;
+        P.work = (unsigned char*)(P.lam + n);
+        P.work = (unsigned char*)(((uintptr_t)P.work + 255) & ~(uintptr_t)255);
+        p = (double*)(((uintptr_t)P.work + eig_work_bytes(n, 64) + 255) & ~(uintptr_t)255);
+        nmax = n > nmax ? n : nmax;
+        kmax = P.k > kmax ? P.k : kmax;
+        fill_gaussian(st, X, (size_t)n * n, 1.0, 555 + t, 6);
+        const std::vector<double> x = down(X, (size_t)n * n);
+        std::vector<double>& g = gs[t];
+        g.assign((size_t)n * n, 0.0);
+        for (int i = 0; i < n; ++i)
+          for (int j = 0; j <= i; ++j) {
+            double s = 0;
+            for (int k = 0; k < n; ++k)
+              s += x[(size_t)i * n + k] * x[(size_t)j * n + k] *
+                   (t % 2 ? (3 * k < n ? 1.0 : 0.0) : std::pow(10.0, -6.0 * k / n));
+            g[(size_t)i * n + j] = g[(size_t)j * n + i] = s;
+          }
+        if (cudaMemcpy(G, g.data(), g.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+          throw std::runtime_error("CUDA error: selftest eig upload");
       }
-      out.push_back(res / gn);
-      out.push_back(orth);
-      out.push_back(order);
+      if (cudaMemcpy(dev.p, probs.data(), np * sizeof(EigProblem), cudaMemcpyHostToDevice) != cudaSuccess)
+        throw std::runtime_error("CUDA error: selftest eig upload");
+      eig_sym_batched(st, (const EigProblem*)dev.p, np, nmax, kmax, 64, err);
+      if (cudaStreamSynchronize(st) != cudaSuccess) throw std::runtime_error("CUDA error: selftest eig");
+      for (int t = 0; t < np; ++t) {
+        const int n = probs[t].n, k = probs[t].k;
+        const std::vector<double> u = down(probs[t].U, (size_t)n * k), lam = down(probs[t].lam, n);
+        double gn = 0, res = 0, orth = 0, order = 0;
+        for (double v : gs[t]) gn = std::fmax(gn, std::fabs(v));
+        for (int c = 1; c < n; ++c)
+          if (lam[c] > lam[c - 1]) order = 1;
+        for (int c = 0; c < k; ++c) {
+          for (int i = 0; i < n; ++i) {
+            double s = 0;
+            for (int q = 0; q < n; ++q) s += gs[t][(size_t)i * n + q] * u[(size_t)q * k + c];
+            const double d = std::fabs(s - lam[c] * u[(size_t)i * k + c]);
+            res = d > res || std::isnan(d) ? d : res;
+          }
+          for (int c2 = 0; c2 < k; ++c2) {
+            double s = 0;
+            for (int q = 0; q < n; ++q) s += u[(size_t)q * k + c] * u[(size_t)q * k + c2];
+            const double d = std::fabs(s - (c == c2 ? 1.0 : 0.0));
+            orth = d > orth || std::isnan(d) ? d : orth;
+          }
+        }
+        out.push_back(res / gn);
+        out.push_back(orth);
+        out.push_back(order);
+      }
     }
   } else if (which == 9) {
     struct Case {

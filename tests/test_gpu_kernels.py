@@ -205,3 +205,12 @@ def test_householder_qr_edges():
         assert o64 < 1e-13 and r64 < 1e-13
         assert o32 < 2e-5 and r32 < 2e-5
         assert ons <= 0.75 * 256 * o32 ** 2 + 2e-12 and rns < 2e-5
+
+
+def test_eigensolver_back_transform_variants():
+    """The largest and smallest sizes of each number of row groups, the variant
+    without registers, mixed sizes in a batch, partial sets of vectors.  The
+    bound is the eigensolver's own."""
+    v = np.array(pkg.qtt_selftest(11)[:-1]).reshape(-1, 3)
+    assert v.shape[0] == 12
+    assert (v[:, :2] < 1e-12).all() and (v[:, 2] == 0).all(), v
