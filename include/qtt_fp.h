@@ -361,7 +361,10 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *      matrix, one with zero and repeated columns and one with graded columns
  *      and rows: as 1, with the residual of the worst column
  *  11  FP64 eigensolver on four batches at the edges of the back-transform's
- *      variants (12 problems): the three values of 2 per problem */
+ *      variants (12 problems): the three values of 2 per problem
+ *  12  two-piece sums of the one-launch GEMM (TF32X3) on operands whose sums
+ *      are exact: per case max |C - C_host|, or -1 where it does not take the
+ *      shape */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

@@ -457,9 +457,10 @@ __global__ void __launch_bounds__(FT, 1) tc_fused_kernel(const FusedArgs g) {
               S += (long long)__float2int_rn(__uint_as_float(v[w][j])) << (8 * (Tr::ngroups - 1 - w));
             bits[j] = int_to_double_bits(S, erow + eb[c0 + j] - 14 - 8 * (Tr::ngroups - 1));
           } else {
-            float f = __uint_as_float(v[0][j]);
-            if (g.pieces == 2) f += __uint_as_float(v[1][j]);
-            bits[j] = float_to_double_bits(__float_as_uint(f));
+            bits[j] = float_to_double_bits(v[0][j]);
+            if (g.pieces == 2)  // the pieces meet in FP64
+              bits[j] = (unsigned long long)__double_as_longlong(
+                  __longlong_as_double((long long)bits[j]) + __longlong_as_double((long long)float_to_double_bits(v[1][j])));
           }
         }
         if (along_rows) {

@@ -41,7 +41,7 @@ bool gemm_tc(cudaStream_t st, int mode, int M, int N, int K, int outer, int inne
 // The same product straight from the FP64 views in one launch (gemm_fused.cu),
 // in the modes TF32X3, BF16X6 and BF16X10, for a tall operand against at most
 // 288 columns; P (TF32X3: up to two pieces) as in small_gemm_sum, the pieces'
-// FP32 sums added in FP32.  False (nothing launched) when the product is not
+// FP32 sums added in FP64.  False (nothing launched) when the product is not
 // of that shape.
 bool gemm_fused(cudaStream_t st, int mode, int M, int N, int K, int outer, int inner, double alpha, MatView A, MatView B,
                 double beta, OutView C, const SumPieces& P, double* ws, size_t ws_elems, int* err);

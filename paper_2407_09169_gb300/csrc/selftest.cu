@@ -83,6 +83,9 @@ std::vector<double> down(const double* d, size_t n) {
 // which = 9: the one-launch tensor-core GEMM against a host sum: per case the
 // mode, the terms of a dot product, max and mean of (C - C_host) / (|alpha|
 // sum |a b| + |beta c0|); -1 where it does not take the shape.
+// which = 12: its two-piece sums on operands whose sums are exact, the second
+// piece 2^-30 of the first: per case max |C - C_host|, -1 where it does not
+// take the shape.
 std::vector<double> run_selftest(int which) {
   cudaStream_t st = nullptr;
   std::vector<double> out;
@@ -758,6 +761,77 @@ std::vector<double> run_selftest(int which) {
           }
       out.push_back(worst);
       out.push_back(mean);
+    }
+  } else if (which == 12) {
+    // Whole numbers of at most 4 in magnitude: products and sums of up to 400
+    // terms are exact in TF32 and FP32, and so is their FP64 sum with 2^-30 of
+    // the same; an FP32 sum of the two pieces keeps none of the second.
+    struct Case {
+      int M, N, K, outer, inner;
+      double alpha, beta;
+    };
+    const Case cases[] = {{128, 136, 77, 5, 1, 1.0, 0.0}, {300, 144, 32, 1, 1, 1.0, 0.0}, {40, 34, 130, 3, 2, -1.0, 1.0}};
+    unsigned int lcg = 1u;
+    auto whole = [&](std::vector<double>& v) {
+      for (double& x : v) {
+        lcg = lcg * 1664525u + 1013904223u;
+        x = (double)((int)(lcg >> 24) % 9 - 4);
+      }
+    };
+    for (const Case& c : cases) {
+      // A [inner][piece][M][K] (no outer index), B [outer][inner][piece][K][N]
+      const long long batch = (long long)c.outer * c.inner;
+      const size_t am = (size_t)c.M * c.K, bm = (size_t)c.K * c.N, cm = (size_t)c.M * c.N;
+      std::vector<double> ha(am * 2 * c.inner), hb(bm * 2 * batch), hc(cm * batch);
+      whole(ha);
+      whole(hb);
+      whole(hc);
+      for (long long b = 0; b < batch; ++b)
+        for (size_t e = 0; e < bm; ++e) hb[(2 * b + 1) * bm + e] *= std::ldexp(1.0, -30);
+      DBuf A(ha.size()), B(hb.size()), C0(hc.size());
+      if (cudaMemcpy(A.p, ha.data(), ha.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemcpy(B.p, hb.data(), hb.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemcpy(C0.p, hc.data(), hc.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess)
+        throw std::runtime_error("CUDA error: selftest upload");
+      MatView av, bv;
+      OutView cv;
+      av.p = A.p;
+      av.rs = c.K;
+      av.cs = 1;
+      av.si = 2 * (long long)am;
+      av.so = 0;
+      bv.p = B.p;
+      bv.rs = c.N;
+      bv.cs = 1;
+      bv.si = 2 * (long long)bm;
+      bv.so = bv.si * c.inner;
+      cv.p = C0.p;
+      cv.rs = c.N;
+      cv.cs = 1;
+      cv.si = (long long)cm;
+      cv.so = cv.si * c.inner;
+      SumPieces P;
+      P.n = 2;
+      P.a = (long long)am;
+      P.b0 = (long long)bm;
+      if (!gemm_fused(st, TC_TF32X3, c.M, c.N, c.K, c.outer, c.inner, c.alpha, av, bv, c.beta, cv, P, nullptr, 0, err)) {
+        out.push_back(-1.0);
+        continue;
+      }
+      const std::vector<double> got = down(C0.p, hc.size());
+      double worst = 0.0;
+      for (long long b = 0; b < batch; ++b)
+        for (int m = 0; m < c.M; ++m)
+          for (int n = 0; n < c.N; ++n) {
+            double v = 0.0;
+            for (int p = 0; p < 2; ++p)
+              for (int k = 0; k < c.K; ++k)
+                v += ha[((b % c.inner) * 2 + p) * am + (size_t)m * c.K + k] * hb[(b * 2 + p) * bm + (size_t)k * c.N + n];
+            const size_t e = (size_t)b * cm + (size_t)m * c.N + n;
+            const double d = std::fabs(got[e] - (c.alpha * v + c.beta * hc[e]));
+            worst = d > worst || std::isnan(d) ? d : worst;
+          }
+      out.push_back(worst);
     }
   } else {
     cudaFree(err);

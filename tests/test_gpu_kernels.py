@@ -214,3 +214,14 @@ def test_eigensolver_back_transform_variants():
     v = np.array(pkg.qtt_selftest(11)[:-1]).reshape(-1, 3)
     assert v.shape[0] == 12
     assert (v[:, :2] < 1e-12).all() and (v[:, 2] == 0).all(), v
+
+
+def test_one_launch_gemm_adds_its_pieces_in_fp64():
+    """Two pieces of whole numbers of at most 4 over at most 130 terms, the
+    second times 2^-30: each piece's sum is exact in TF32 products and an FP32
+    accumulator (below 2^12), their sum and the beta term fit 53 bits, so the
+    result is the host's sum exactly.  An FP32 sum of the pieces loses the
+    second one."""
+    v = np.array(pkg.qtt_selftest(12))
+    assert v[-1] == 0, "a bounded wait gave up"
+    assert v[:-1].tolist() == [0.0, 0.0, 0.0]
