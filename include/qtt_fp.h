@@ -364,7 +364,9 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *      variants (12 problems): the three values of 2 per problem
  *  12  two-piece sums of the one-launch GEMM (TF32X3) on operands whose sums
  *      are exact: per case max |C - C_host|, or -1 where it does not take the
- *      shape */
+ *      shape
+ *  13  (needs no GPU) the measures of 1 and 10 on an exact Q, on one with a NaN
+ *      and on one of NaN: max |Q^T Q - I|, residual, residual of the worst column */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

@@ -63,6 +63,41 @@ std::vector<double> down(const double* d, size_t n) {
     throw std::runtime_error("CUDA error: selftest copy");
   return h;
 }
+// The larger of the worst value so far and d, a NaN once there is one (std::fmax would drop it).
+double worse(double worst, double d) { return d > worst || std::isnan(d) ? d : worst; }
+
+// Of Q (m x n, row-major): max |Q^T Q - I|, ||Y - Q Q^T Y||_F / ||Y||_F and the
+// same of the worst column.
+struct QrErrors {
+  double orth, resid, worst;
+};
+QrErrors qr_errors(int m, int n, const std::vector<double>& y, const std::vector<double>& q) {
+  QrErrors e{0, 0, 0};
+  for (int a = 0; a < n; ++a)
+    for (int b = 0; b < n; ++b) {
+      double s = 0;
+      for (int i = 0; i < m; ++i) s += q[(size_t)i * n + a] * q[(size_t)i * n + b];
+      e.orth = worse(e.orth, std::fabs(s - (a == b ? 1.0 : 0.0)));
+    }
+  double num = 0, den = 0;
+  for (int c = 0; c < n; ++c) {
+    std::vector<double> coef(n, 0.0);
+    double cn = 0, cd = 0;
+    for (int a = 0; a < n; ++a)
+      for (int i = 0; i < m; ++i) coef[a] += q[(size_t)i * n + a] * y[(size_t)i * n + c];
+    for (int i = 0; i < m; ++i) {
+      double r = y[(size_t)i * n + c];
+      for (int a = 0; a < n; ++a) r -= q[(size_t)i * n + a] * coef[a];
+      cn += r * r;
+      cd += y[(size_t)i * n + c] * y[(size_t)i * n + c];
+    }
+    num += cn;
+    den += cd;
+    if (cd > 0) e.worst = worse(e.worst, std::sqrt(cn / cd));
+  }
+  e.resid = std::sqrt(num / den);
+  return e;
+}
 }  // namespace
 
 // which = 0: tensor-core GEMM modes against the FP64 GEMM.  For every case
@@ -86,7 +121,23 @@ std::vector<double> down(const double* d, size_t n) {
 // which = 12: its two-piece sums on operands whose sums are exact, the second
 // piece 2^-30 of the first: per case max |C - C_host|, -1 where it does not
 // take the shape.
+// which = 13 (no GPU): the QR measures of 1 and 10 on an exact Q, one with a
+// NaN and one of NaN: orthonormality, residual, worst column's residual.
 std::vector<double> run_selftest(int which) {
+  if (which == 13) {
+    // Q = the first n columns of I and Y = Q: exact, one NaN in Q, Q all NaN
+    const int m = 5, n = 3;
+    std::vector<double> q((size_t)m * n, 0.0), v;
+    for (int i = 0; i < n; ++i) q[(size_t)i * n + i] = 1.0;
+    const std::vector<double> y = q;
+    for (int kind = 0; kind < 3; ++kind) {
+      if (kind == 1) q[4 * n + 1] = std::nan("");
+      if (kind == 2) q.assign(q.size(), std::nan(""));
+      const QrErrors e = qr_errors(m, n, y, q);
+      v.insert(v.end(), {e.orth, e.resid, e.worst});
+    }
+    return v;
+  }
   cudaStream_t st = nullptr;
   std::vector<double> out;
   int* err = nullptr;
@@ -149,7 +200,7 @@ std::vector<double> run_selftest(int which) {
         double mx = 0, md = 0;
         for (size_t i = 0; i < csz; ++i) {
           mx = std::fmax(mx, std::fabs(h0[i]));
-          md = std::fmax(md, std::fabs(h0[i] - h1[i]));
+          md = worse(md, std::fabs(h0[i] - h1[i]));
         }
         out.push_back(md / (mx > 0 ? mx : 1.0));
       }
@@ -194,32 +245,9 @@ std::vector<double> run_selftest(int which) {
           }
           if (cudaStreamSynchronize(st) != cudaSuccess) throw std::runtime_error("CUDA error: selftest qr");
           std::vector<double> q = down(Q.p, (size_t)m * n);
-          double orth = 0;
-          for (int a = 0; a < n; ++a)
-            for (int b2 = 0; b2 < n; ++b2) {
-              double s = 0;
-              for (int i = 0; i < m; ++i) s += q[(size_t)i * n + a] * q[(size_t)i * n + b2];
-              orth = std::fmax(orth, std::fabs(s - (a == b2 ? 1.0 : 0.0)));
-            }
-          // projection residual ||Y - Q Q^T Y||_F / ||Y||_F, or of the worst column
-          double num = 0, den = 0, worst = 0;
-          for (int c = 0; c < n; ++c) {
-            std::vector<double> coef(n, 0.0);
-            double cn = 0, cd = 0;
-            for (int a = 0; a < n; ++a)
-              for (int i = 0; i < m; ++i) coef[a] += q[(size_t)i * n + a] * y[(size_t)i * n + c];
-            for (int i = 0; i < m; ++i) {
-              double r = y[(size_t)i * n + c];
-              for (int a = 0; a < n; ++a) r -= q[(size_t)i * n + a] * coef[a];
-              cn += r * r;
-              cd += y[(size_t)i * n + c] * y[(size_t)i * n + c];
-            }
-            num += cn;
-            den += cd;
-            if (cd > 0) worst = std::fmax(worst, std::sqrt(cn / cd));
-          }
-          out.push_back(orth);
-          out.push_back(which == 1 ? std::sqrt(num / den) : worst);
+          const QrErrors e = qr_errors(m, n, y, q);
+          out.push_back(e.orth);
+          out.push_back(which == 1 ? e.resid : e.worst);
         }
       }
   } else if (which == 2) {
@@ -277,12 +305,12 @@ std::vector<double> run_selftest(int which) {
           for (int i = 0; i < n; ++i) {
             double s = 0;
             for (int k = 0; k < n; ++k) s += g[(size_t)i * n + k] * u[(size_t)k * n + c];
-            res = std::fmax(res, std::fabs(s - lam[c] * u[(size_t)i * n + c]));
+            res = worse(res, std::fabs(s - lam[c] * u[(size_t)i * n + c]));
           }
           for (int c2 = 0; c2 < n; ++c2) {
             double s = 0;
             for (int k = 0; k < n; ++k) s += u[(size_t)k * n + c] * u[(size_t)k * n + c2];
-            orth = std::fmax(orth, std::fabs(s - (c == c2 ? 1.0 : 0.0)));
+            orth = worse(orth, std::fabs(s - (c == c2 ? 1.0 : 0.0)));
           }
         }
         out.push_back(res / gn);
@@ -329,7 +357,7 @@ std::vector<double> run_selftest(int which) {
           for (size_t i = 0; i < h0.size(); ++i) {
             const double r = (h1[i] - h0[i]) / h0[i];
             mean += r;
-            mx = std::fmax(mx, std::fabs(r));
+            mx = worse(mx, std::fabs(r));
           }
           out.push_back(mean / (double)h0.size());
           out.push_back(mx);
@@ -393,7 +421,7 @@ std::vector<double> run_selftest(int which) {
               ref += ar[k] * bc[k];
               mag += std::fabs(ar[k] * bc[k]);
             }
-            err_max = std::fmax(err_max, std::fabs(cij - ref) / mag);
+            err_max = worse(err_max, std::fabs(cij - ref) / mag);
           }
         }
         out.push_back((double)n);
@@ -593,7 +621,7 @@ std::vector<double> run_selftest(int which) {
             const double ref = c.alpha * v + c.beta * hc[e];
             const double scale = std::fabs(c.alpha) * mag + std::fabs(c.beta * hc[e]);
             const double d = std::fabs(got[e] - ref) / scale;
-            worst = d > worst || std::isnan(d) ? d : worst;
+            worst = worse(worst, d);
           }
       out.push_back((double)c.kind);
       out.push_back((double)c.K * c.pieces);
@@ -660,13 +688,13 @@ std::vector<double> run_selftest(int which) {
             double s = 0;
             for (int q = 0; q < n; ++q) s += gs[t][(size_t)i * n + q] * u[(size_t)q * k + c];
             const double d = std::fabs(s - lam[c] * u[(size_t)i * k + c]);
-            res = d > res || std::isnan(d) ? d : res;
+            res = worse(res, d);
           }
           for (int c2 = 0; c2 < k; ++c2) {
             double s = 0;
             for (int q = 0; q < n; ++q) s += u[(size_t)q * k + c] * u[(size_t)q * k + c2];
             const double d = std::fabs(s - (c == c2 ? 1.0 : 0.0));
-            orth = d > orth || std::isnan(d) ? d : orth;
+            orth = worse(orth, d);
           }
         }
         out.push_back(res / gn);
@@ -756,7 +784,7 @@ std::vector<double> run_selftest(int which) {
             }
             const size_t e = (size_t)b * cm + (c.flip_c ? (size_t)n * c.M + m : (size_t)m * c.N + n);
             const double d = (got[e] - c.alpha * v - c.beta * hc[e]) / (std::fabs(c.alpha) * mag + std::fabs(c.beta * hc[e]));
-            worst = std::fabs(d) > worst || std::isnan(d) ? std::fabs(d) : worst;
+            worst = worse(worst, std::fabs(d));
             mean += d / ((double)cm * batch);
           }
       out.push_back(worst);
@@ -829,7 +857,7 @@ std::vector<double> run_selftest(int which) {
                 v += ha[((b % c.inner) * 2 + p) * am + (size_t)m * c.K + k] * hb[(b * 2 + p) * bm + (size_t)k * c.N + n];
             const size_t e = (size_t)b * cm + (size_t)m * c.N + n;
             const double d = std::fabs(got[e] - (c.alpha * v + c.beta * hc[e]));
-            worst = d > worst || std::isnan(d) ? d : worst;
+            worst = worse(worst, d);
           }
       out.push_back(worst);
     }

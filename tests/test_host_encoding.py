@@ -251,3 +251,11 @@ def test_subgrid_rejects_large_grids_and_bad_constants():
     p = _sgs([2, 2, 2, 2, 2], c_omega=-1.0)
     with pytest.raises(pkg.QttError):
         pkg.qtt_host_dense(p, 40, 64)
+
+
+def test_qr_self_check_measures_report_nan():
+    """The measures that the QR self-checks return: zero for an exact Q, NaN
+    as soon as an entry of Q is (a maximum that drops NaN would pass it)."""
+    v = pkg.qtt_selftest(13).reshape(3, 3)
+    assert (v[0] == 0.0).all()
+    assert np.isnan(v[1:]).all(), v
