@@ -235,8 +235,9 @@ qtt_status qtt_truncate_vjp(int32_t N, const int32_t* rx, const double* x, const
  * (after its first three steps), each step is one launch of a graph that
  * embeds every context's step graph as an independent node; it is built the
  * first time a set of contexts is stepped together, kept for the four sets
- * stepped last, and rebuilt when a context's graphs or the contexts' relative
- * step parity change (the contexts must belong to the current device).  The
+ * stepped last until one of their contexts is destroyed, and rebuilt when a
+ * context's graphs or the contexts' relative step parity change (the contexts
+ * must belong to the current device).  The
  * contexts may differ in grid, chi, coefficients and precision; a context
  * must not appear twice.  Returns QTT_OK, or the status of the first context
  * (lowest index) that failed, whose index goes to *failed (-1 when none;
@@ -366,7 +367,10 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *      are exact: per case max |C - C_host|, or -1 where it does not take the
  *      shape
  *  13  (needs no GPU) the measures of 1 and 10 on an exact Q, on one with a NaN
- *      and on one of NaN: max |Q^T Q - I|, residual, residual of the worst column */
+ *      and on one of NaN: max |Q^T Q - I|, residual, residual of the worst column
+ *  14  (needs no GPU) bookkeeping of qtt_step_many: the sets of contexts whose
+ *      parent graphs are kept, the destroyed contexts whose sets are still to
+ *      be dropped */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

@@ -251,7 +251,9 @@ namespace {
 // them takes longer than several steps, so the graphs of the last kBatchSets
 // sets are kept: four steps of a set of 12, three sets in turn, take 239 ms
 // where rebuilding at every change of the set made it 463.  A set is dropped
-// when one of its contexts is destroyed.
+// when one of its contexts is destroyed; while a batch call holds the sets,
+// qtt_destroy (which does not wait for it) only notes the context's id, and
+// that call drops the set when it lets go.
 constexpr size_t kBatchSets = 4;
 struct BatchGraph {
   std::vector<unsigned long long> ids;
@@ -271,7 +273,7 @@ std::vector<BatchGraph> g_batch;              // most recently used first
 cudaStream_t g_batch_st = nullptr;
 cudaEvent_t g_batch_ev = nullptr;
 std::vector<cudaEvent_t> g_batch_ctx_ev;
-std::mutex g_dead_mu;                         // qtt_destroy only notes the id
+std::mutex g_dead_mu;
 std::vector<unsigned long long> g_dead_ids;
 std::atomic<bool> g_batch_used{false};
 
@@ -281,7 +283,7 @@ void batch_note_destroyed(unsigned long long id) {
   g_dead_ids.push_back(id);
 }
 
-// drops the sets that hold a destroyed context
+// drops the sets that hold a destroyed context (g_batch_mu held)
 void batch_purge() {
   std::vector<unsigned long long> dead;
   {
@@ -299,6 +301,29 @@ void batch_purge() {
     }
   }
 }
+
+size_t batch_noted() {
+  std::lock_guard<std::mutex> lk(g_dead_mu);
+  return g_dead_ids.size();
+}
+
+// The same from a thread that does not hold g_batch_mu.  Whoever holds it
+// comes through here after unlocking, so an id noted meanwhile is not left.
+void batch_collect() {
+  while (batch_noted() > 0) {
+    std::unique_lock<std::mutex> lk(g_batch_mu, std::try_to_lock);
+    if (!lk.owns_lock()) return;
+    batch_purge();
+  }
+}
+struct BatchCollector {
+  ~BatchCollector() {
+    try {
+      batch_collect();
+    } catch (...) {
+    }
+  }
+};
 
 bool batch_build(qtt_ctx* const* ctxs, int32_t n) {
   if (!g_batch_st && cudaStreamCreateWithFlags(&g_batch_st, cudaStreamNonBlocking) != cudaSuccess) return false;
@@ -390,6 +415,7 @@ qtt_status qtt_step_many(qtt_ctx* const* ctxs, int32_t n, int32_t nsteps, int32_
   // step-major order: every context's step s is enqueued before any step s+1
   std::vector<int> bad(n, 0);
   std::vector<qtt_status> code(n, QTT_OK);
+  BatchCollector collector;  // runs after the lock is released
   std::lock_guard<std::mutex> batch_lock(g_batch_mu);
   batch_purge();
   bool on_batch = false;  // the batch stream holds work the contexts' streams have not waited for
@@ -708,6 +734,7 @@ void qtt_destroy(qtt_ctx* ctx) {
     if (ctx->eng) {
       cudaStreamSynchronize(ctx->eng->stream());
       batch_note_destroyed(ctx->eng->id());
+      batch_collect();
     }
   } catch (...) {
   }
@@ -850,6 +877,10 @@ qtt_status qtt_truncate_vjp(int32_t N, const int32_t* rx, const double* x, const
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written) {
   if (written) *written = 0;
   try {
+    if (which == 14) {
+      std::lock_guard<std::mutex> lk(g_batch_mu);
+      return put({(double)g_batch.size(), (double)batch_noted()}, out, cap, written);
+    }
     int ndev = 0;
     if (which != 13 && (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0)) {
       cudaGetLastError();

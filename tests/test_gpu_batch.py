@@ -90,3 +90,27 @@ def test_sets_stepped_in_turn_match_separate_steps():
             c.close()
         for c in alone:
             c.close()
+
+
+def test_parent_graphs_go_with_their_contexts():
+    """The parent graphs of a set are dropped when one of its contexts is
+    destroyed, without another batch call, and no destroyed context stays
+    noted; a set that does not hold it stays."""
+    kept = lambda: pkg.qtt_selftest(14).tolist()
+    ps = _instances()[:2]
+    before = kept()[0]
+    a, b = [pkg.qtt_init(p) for p in ps], [pkg.qtt_init(p) for p in ps]
+    try:
+        pkg.qtt_step_many(a, 4)
+        pkg.qtt_step_many(b, 4)
+        assert kept() == [before + 2, 0]
+        a[0].close()
+        assert kept() == [before + 1, 0]
+        b[1].close()
+        assert kept() == [before, 0]
+        a[1].close()
+        pkg.qtt_init(ps[0]).close()
+        assert kept() == [before, 0]
+    finally:
+        for c in a + b:
+            c.close()
