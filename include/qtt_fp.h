@@ -247,7 +247,11 @@ qtt_status qtt_step_many(qtt_ctx* const* ctxs, int32_t n, int32_t nsteps, int32_
 
 /* Extract observables (see qtt_observable).  `out` has room for `cap`
  * doubles; *written receives the number written.  Returns QTT_EINVAL when
- * cap is too small. */
+ * cap is too small.  The device scratch of the dense, mean-field, point and
+ * error observables (4 doubles per dense value or per value of the three mean
+ * fields) is one buffer per device up to 64 MB, kept for all contexts until
+ * the last one is destroyed; a larger request, or one made while another
+ * thread's call uses the buffer, allocates and frees its own. */
 qtt_status qtt_observe(qtt_ctx* ctx, int32_t what, double* out, int64_t cap, int64_t* written);
 
 /* Relative L2 distance ||a - b|| / ||b|| of the two states (same grid),

@@ -35,6 +35,8 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <stdexcept>
 #include <string>
 
@@ -189,7 +191,6 @@ Engine::~Engine() {
   for (cudaGraph_t& g : graph_tmpl_)
     if (g) cudaGraphDestroy(g);
   for (void* a : allocs_) cudaFree(a);
-  if (obs_buf_) cudaFree(obs_buf_);
   for (void* w : pack_ws_)
     if (w) cudaFree(w);
   for (int l = 1; l < kLanes; ++l) {
@@ -1109,29 +1110,86 @@ void Engine::scalars(double out[13]) {
   out[12] = n2;  // sum of f^2 over every grid cell
 }
 
-Engine::Scratch::Scratch(Engine& e, size_t bytes) : eng(e) {
-  if (bytes <= kObsKeep && !e.obs_busy_) {
-    if (bytes > e.obs_bytes_) {
-      if (e.obs_buf_) {
-        QTT_CUDA(cudaStreamSynchronize(e.st_));
-        QTT_CUDA(cudaFree(e.obs_buf_));
-      }
-      e.obs_buf_ = nullptr;
-      e.obs_bytes_ = 0;
-      QTT_CUDA(cudaMalloc(&e.obs_buf_, bytes));
-      e.obs_bytes_ = bytes;
-    }
-    e.obs_busy_ = true;
-    kept = true;
-    p = (unsigned char*)e.obs_buf_;
-  } else {
-    QTT_CUDA(cudaMalloc(&p, bytes));
+namespace {
+struct ObsPool {
+  struct Dev {
+    void* p = nullptr;
+    size_t bytes = 0;
+    bool busy = false;
+    int users = 0;
+  };
+  std::mutex mu;
+  std::map<int, Dev> dev;
+};
+ObsPool& obs_pool() {
+  static ObsPool* pool = new ObsPool;  // outlives every engine
+  return *pool;
+}
+}  // namespace
+
+ObsUser::ObsUser() {
+  int d = -1;
+  if (cudaGetDevice(&d) != cudaSuccess) {
+    cudaGetLastError();
+    return;
   }
+  ObsPool& pool = obs_pool();
+  std::lock_guard<std::mutex> lk(pool.mu);
+  ++pool.dev[d].users;
+  dev_ = d;
+}
+
+ObsUser::~ObsUser() {
+  if (dev_ < 0) return;
+  ObsPool& pool = obs_pool();
+  std::lock_guard<std::mutex> lk(pool.mu);
+  ObsPool::Dev& d = pool.dev[dev_];
+  if (--d.users > 0 || !d.p) return;
+  cudaFree(d.p);
+  d.p = nullptr;
+  d.bytes = 0;
+}
+
+void* ObsUser::take(size_t bytes) {
+  if (dev_ < 0 || bytes > kObsKeep) return nullptr;
+  ObsPool& pool = obs_pool();
+  std::lock_guard<std::mutex> lk(pool.mu);
+  ObsPool::Dev& d = pool.dev[dev_];
+  if (d.busy) return nullptr;
+  if (bytes > d.bytes) {
+    if (d.p) cudaFree(d.p);  // not busy: no work in flight uses it
+    d.p = nullptr;
+    d.bytes = 0;
+    if (cudaMalloc(&d.p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      d.p = nullptr;
+      return nullptr;
+    }
+    d.bytes = bytes;
+  }
+  d.busy = true;
+  return d.p;
+}
+
+void ObsUser::give() {
+  ObsPool& pool = obs_pool();
+  std::lock_guard<std::mutex> lk(pool.mu);
+  pool.dev[dev_].busy = false;
+}
+
+Engine::Scratch::Scratch(Engine& e, size_t bytes) : eng(e) {
+  p = (unsigned char*)e.obs_user_.take(bytes);
+  kept = p != nullptr;
+  if (!kept) QTT_CUDA(cudaMalloc(&p, bytes));
 }
 
 Engine::Scratch::~Scratch() {
-  if (kept) eng.obs_busy_ = false;
-  else if (p) cudaFree(p);
+  if (kept) {
+    cudaStreamSynchronize(eng.st_);  // the callers wait for their results; an exception may leave before
+    eng.obs_user_.give();
+  } else if (p) {
+    cudaFree(p);
+  }
 }
 
 size_t Engine::chain_dense_bytes(size_t rows) { return sizeof(double) * (rows + 16) * 4; }

@@ -114,6 +114,26 @@ inline OutView ov(double* p, long long rs, long long cs, long long so = 0, long 
 
 struct KernelTimer;
 
+// An engine's share in the scratch that the observable calls of a device keep
+// between them: one buffer of at most kObsKeep bytes for all engines of the
+// device, as large as the largest such request so far, taken by one call at a
+// time (others allocate their own meanwhile) and freed with the device's last
+// engine.  An allocation per call costs about as much as the observables of a
+// small state; a buffer per engine would hold 64 MB for each of an ensemble.
+class ObsUser {
+ public:
+  static constexpr size_t kObsKeep = (size_t)64 << 20;
+  ObsUser();
+  ~ObsUser();
+  ObsUser(const ObsUser&) = delete;
+  ObsUser& operator=(const ObsUser&) = delete;
+  void* take(size_t bytes);  // null: in use, too large, or no memory
+  void give();               // nothing on the device may still use the buffer
+
+ private:
+  int dev_ = -1;
+};
+
 class Engine {
  public:
   explicit Engine(const Params& p, cudaStream_t stream);
@@ -223,10 +243,8 @@ class Engine {
   void grad_terms(const DevMps& a, const DevMps& f, const double* hf, double w);
   void set_step_counter(unsigned long long s);
 
-  // Device scratch of one observable call: the engine's kept buffer up to
-  // kObsKeep bytes (it grows with the requests and goes with the engine), an
-  // allocation of its own above that.
-  static constexpr size_t kObsKeep = (size_t)64 << 20;
+  // Device scratch of one observable call: the device's kept buffer (see
+  // ObsUser) where it is free, else an allocation of its own.
   struct Scratch {
     Engine& eng;
     unsigned char* p = nullptr;
@@ -236,9 +254,7 @@ class Engine {
     Scratch(const Scratch&) = delete;
     Scratch& operator=(const Scratch&) = delete;
   };
-  void* obs_buf_ = nullptr;
-  size_t obs_bytes_ = 0;
-  bool obs_busy_ = false;
+  ObsUser obs_user_;
 
   Params p_;
   Model model_;

@@ -378,3 +378,36 @@ def test_point_blocks_match_dense(npts):
         vals = ctx.points(idx)
     # 15 sites of at most 45 terms each in another order: far below 1e-13 of the largest value
     assert np.abs(vals - dense[tuple(idx.T)]).max() <= 1e-13 * np.abs(dense).max()
+
+
+def test_observable_scratch_is_shared_by_the_contexts():
+    """Dense read-backs of 2^20 values use 33.5 MB of scratch: one buffer for
+    all contexts of the device (eight contexts after the first add nothing; a
+    buffer for each would add 268 MB), the same values from several threads at
+    once, and given back with the last context."""
+    import gc
+    from concurrent.futures import ThreadPoolExecutor
+
+    import torch
+
+    gc.collect()
+    p = workload.make_params("small")
+    p["chi_max"] = 6
+    ctxs = [pkg.qtt_init(dict(p, seed=i)) for i in range(9)]
+    try:
+        dense = lambda c: c.observe(pkg.OBS_DENSE)
+        first = dense(ctxs[0])
+        free = torch.cuda.mem_get_info()[0]
+        ref = [first] + [dense(c) for c in ctxs[1:]]
+        assert free - torch.cuda.mem_get_info()[0] <= 16 << 20
+        with ThreadPoolExecutor(4) as ex:
+            for got, want in zip(ex.map(dense, ctxs * 3), ref * 3):
+                assert np.array_equal(got, want)
+        assert free - torch.cuda.mem_get_info()[0] <= 16 << 20
+        for c in ctxs[1:]:
+            c.close()
+        free = torch.cuda.mem_get_info()[0]
+    finally:
+        for c in ctxs:
+            c.close()
+    assert torch.cuda.mem_get_info()[0] - free >= 33 << 20
