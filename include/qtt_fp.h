@@ -374,7 +374,11 @@ qtt_status qtt_host_dense(const qtt_params* params, int32_t which, double* out, 
  *      and on one of NaN: max |Q^T Q - I|, residual, residual of the worst column
  *  14  (needs no GPU) bookkeeping of qtt_step_many: the sets of contexts whose
  *      parent graphs are kept, the destroyed contexts whose sets are still to
- *      be dropped */
+ *      be dropped
+ *  15  the one-launch GEMM at the limits of K and on graded operands: per case
+ *      the mode's enum value, K, the kind of operands (0 Gaussian, 1 graded
+ *      over decades, 2 with zeros) and max |C - C_host| / sum |a b|, or -1
+ *      where it does not take the shape */
 qtt_status qtt_selftest(int32_t which, double* out, int64_t cap, int64_t* written);
 
 #ifdef __cplusplus

@@ -44,6 +44,7 @@ namespace {
 constexpr int FT = 512;          // threads: 16 warps
 constexpr int FW = FT / 32;
 constexpr int FK_MAX = 512;      // K of one exact-slice product (its shifts sit in shared memory)
+constexpr int kAbsent = 4096;    // a shift that takes every value below the smallest one
 
 template <int MODE>
 struct FusedTraits;
@@ -123,8 +124,8 @@ __device__ __forceinline__ void cut(double x, int c, uint32_t* s) {
     const int E = (int)(hi >> 20) & 0x7FF;
     const uint32_t m = (hi & 0xFFFFFu) | 0x100000u;
     // (m, lo) >> (sh - 1), sh = 52 - (E - 1023 + 8 ns - 1 - c) >= 53 - (8 ns - 1)
-    const int t = 1075 - 8 * ns + c - E;  // sh - 1
-    uint32_t v = t < 32 ? __funnelshift_r(lo, m, (uint32_t)t) : (t < 64 ? m >> (t - 32) : 0u);
+    const uint32_t t = (uint32_t)(1075 - 8 * ns + c - E);  // sh - 1; a zero under kAbsent wraps to the last case
+    uint32_t v = t < 32 ? __funnelshift_r(lo, m, t) : (t < 64 ? m >> (t - 32) : 0u);
     if (E == 0) v = 0u;
     const uint32_t rest = t < 32 ? lo << (32 - t) : (lo | (t > 32 && t < 64 ? m << (64 - t) : 0u));  // below the half
     uint32_t u = (v >> 1) + (v & (rest ? 1u : (v >> 1)) & 1u);
@@ -339,14 +340,16 @@ __global__ void __launch_bounds__(FT, 1) tc_fused_kernel(const FusedArgs g) {
     // K index shifts: half the difference of the two operands' largest
     // exponents at k, so that both carry the square root of the terms' sizes
     // and the terms far below the largest one keep the same relative
-    // accuracy in either operand
+    // accuracy in either operand.  A k that is zero in one operand adds
+    // nothing: it leaves the other one too, whose scales it would otherwise
+    // set (1e9 there against balanced terms around 1 left no correct digit)
     for (int k = tid; k < nk; k += FT) {
       int ma = 0, mb = 0;
 #pragma unroll 8
       for (int n = 0; n < cols; ++n) mb = max(mb, (int)tb[k * PB + n]);
 #pragma unroll 8
       for (int r = 0; r < rows; ++r) ma = max(ma, (int)ta[k * PA + r]);
-      ksh[k] = (ma == 0 || mb == 0) ? 0 : (mb - ma) >> 1;
+      ksh[k] = ma == 0 ? kAbsent : mb == 0 ? -kAbsent : (mb - ma) >> 1;
     }
     __syncthreads();
     row_fields<BM>(ta, PA, rows, nk, ksh, 1, ea);

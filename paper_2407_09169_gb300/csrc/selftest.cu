@@ -121,6 +121,10 @@ QrErrors qr_errors(int m, int n, const std::vector<double>& y, const std::vector
 // which = 12: its two-piece sums on operands whose sums are exact, the second
 // piece 2^-30 of the first: per case max |C - C_host|, -1 where it does not
 // take the shape.
+// which = 15: the one-launch tensor-core GEMM at the limits of K and on graded
+// operands: per case the mode, K, the kind (0 Gaussian, 1 graded, 2 graded with
+// zeros) and max |C - C_host| / sum |a b| (0 / 0 counts as 0), -1 where it does
+// not take the shape.
 // which = 13 (no GPU): the QR measures of 1 and 10 on an exact Q, one with a
 // NaN and one of NaN: orthonormality, residual, worst column's residual.
 std::vector<double> run_selftest(int which) {
@@ -859,6 +863,84 @@ std::vector<double> run_selftest(int which) {
             const double d = std::fabs(got[e] - (c.alpha * v + c.beta * hc[e]));
             worst = worse(worst, d);
           }
+      out.push_back(worst);
+    }
+  } else if (which == 15) {
+    struct Case {
+      int mode, M, N, K;
+      bool ta, tb;
+      int kind;
+    };
+    // the largest K of the exact-slice modes and one more; both layouts of either operand
+    const Case cases[] = {
+        {TC_BF16X10, 150, 136, 448, false, false, 0}, {TC_BF16X10, 150, 70, 449, false, false, 0},
+        {TC_BF16X10, 150, 70, 300, true, false, 1},   {TC_BF16X10, 131, 136, 300, false, true, 2},
+        {TC_BF16X6, 150, 144, 352, false, false, 0},  {TC_BF16X6, 150, 144, 353, false, false, 0},
+        {TC_BF16X6, 150, 70, 330, true, false, 1},    {TC_BF16X6, 131, 140, 330, false, true, 2},
+        {TC_TF32X3, 150, 144, 330, false, false, 1},  {TC_TF32X3, 131, 140, 330, true, true, 2}};
+    unsigned long long seed = 1357;
+    for (const Case& c : cases) {
+      const int M = c.M, N = c.N, K = c.K;
+      const size_t am = (size_t)M * K, bm = (size_t)K * N, cm = (size_t)M * N;
+      DBuf A(am), B(bm), C0(cm);
+      fill_gaussian(st, A.p, am, 1.0, seed++, 1);
+      fill_gaussian(st, B.p, bm, 1.0, seed++, 2);
+      std::vector<double> ha = down(A.p, am), hb = down(B.p, bm);
+      auto a = [&](int m, int k) -> double& { return ha[c.ta ? (size_t)k * M + m : (size_t)m * K + k]; };
+      auto b = [&](int k, int n) -> double& { return hb[c.tb ? (size_t)n * K + k : (size_t)k * N + n]; };
+      if (c.kind > 0) {
+        // column k of A times 10^(-12, 0, 12), row k of B by the inverse; rows of A
+        // and columns of B over decades; entries 10^-8 and 10^-30 of their neighbours
+        for (int k = 0; k < K; ++k) {
+          const double g = std::pow(10.0, 12 * (k % 3 - 1));
+          for (int m = 0; m < M; ++m)
+            a(m, k) *= g * std::pow(10.0, 6 * (m % 5 - 2)) * ((m + k) % 7 == 0 ? 1e-8 : (m + k) % 7 == 1 ? 1e-30 : 1.0);
+          for (int n = 0; n < N; ++n) b(k, n) *= std::pow(10.0, 5 * (n % 3 - 1)) / g;
+        }
+      }
+      if (c.kind == 2) {
+        // zero rows and columns; K indices that are zero in A, in B (large in the other operand) and in both
+        for (int k = 0; k < K; ++k)
+          for (int m = 0; m < M; ++m)
+            if (m % 41 == 3 || k % 29 == 5 || k % 29 == 7) a(m, k) = 0.0;
+            else if (k % 29 == 6) a(m, k) = 1e9 * (1.0 + m % 3);
+        for (int k = 0; k < K; ++k)
+          for (int n = 0; n < N; ++n)
+            if (n % 37 == 2 || k % 29 == 6 || k % 29 == 7) b(k, n) = 0.0;
+            else if (k % 29 == 5) b(k, n) = 1e9 * (1.0 + n % 3);
+      }
+      if (cudaMemcpy(A.p, ha.data(), am * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
+          cudaMemcpy(B.p, hb.data(), bm * 8, cudaMemcpyHostToDevice) != cudaSuccess)
+        throw std::runtime_error("CUDA error: selftest upload");
+      MatView av, bv;
+      OutView cv;
+      av.p = A.p;
+      av.rs = c.ta ? 1 : K;
+      av.cs = c.ta ? M : 1;
+      bv.p = B.p;
+      bv.rs = c.tb ? 1 : N;
+      bv.cs = c.tb ? K : 1;
+      cv.p = C0.p;
+      cv.rs = N;
+      cv.cs = 1;
+      out.insert(out.end(), {(double)c.mode, (double)K, (double)c.kind});
+      if (!gemm_fused(st, c.mode, M, N, K, 1, 1, 1.0, av, bv, 0.0, cv, SumPieces{}, nullptr, 0, err)) {
+        out.push_back(-1.0);
+        continue;
+      }
+      const std::vector<double> got = down(C0.p, cm);
+      double worst = 0.0;
+      for (int m = 0; m < M; ++m)
+        for (int n = 0; n < N; ++n) {
+          double v = 0.0, mag = 0.0;
+          for (int k = 0; k < K; ++k) {
+            const double t = a(m, k) * b(k, n);
+            v += t;
+            mag += std::fabs(t);
+          }
+          const double d = std::fabs(got[(size_t)m * N + n] - v);
+          worst = worse(worst, d == 0.0 ? 0.0 : d / mag);
+        }
       out.push_back(worst);
     }
   } else {

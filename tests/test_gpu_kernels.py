@@ -225,3 +225,29 @@ def test_one_launch_gemm_adds_its_pieces_in_fp64():
     v = np.array(pkg.qtt_selftest(12))
     assert v[-1] == 0, "a bounded wait gave up"
     assert v[:-1].tolist() == [0.0, 0.0, 0.0]
+
+
+def test_one_launch_gemm_graded_operands():
+    """K at the largest of the exact-slice modes (one more is refused), and
+    operands whose K indices, rows and columns span decades, with entries far
+    below their row's largest, zero rows and columns, and K indices that are
+    zero in one operand and large in the other (they add nothing to any sum, so
+    they may not cost the other terms precision).  Bounds as in
+    test_one_launch_tensor_core_gemm; the K shifts are whole powers of two from
+    whole exponents, within (-1, 1/2] of the balance, so on graded operands a K
+    index can stand 2^1.5 above the others in one operand: a factor of 4."""
+    v = np.array(pkg.qtt_selftest(15))
+    assert v[-1] == 0, "a bounded wait gave up"
+    v = v[:-1].reshape(-1, 4)
+    assert v.shape[0] == 10
+    limit = {"bf16x6": 352, "bf16x10": 448}
+    for mode, K, kind, worst in v:
+        m = MODES[int(mode)]
+        if m in limit and K > limit[m]:
+            assert worst == -1, (m, K)
+            continue
+        bound = {"tf32x3": 3 * 2.0 ** -22 + (K / 8) * 2.0 ** -23, "bf16x6": 4.5e-6, "bf16x10": 4.5e-6 * 2.0 ** -7}[m]
+        if kind > 0 and m != "tf32x3":
+            bound *= 4
+        print(f"{m} K {int(K)} kind {int(kind)}: {worst:.2e} (bound {bound:.1e})")
+        assert 0 <= worst <= bound, (m, K, kind, worst)
