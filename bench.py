@@ -428,7 +428,7 @@ def run_mine(args, rank, world, local_rank):
             peak = bf16 / passes
             ach = g["gflop_per_step"] / (g["ms_per_step"] / 1e3) / 1e3 if g["ms_per_step"] > 0 else 0.0
             roofline = {
-                "kernel": "gemm_tc (tcgen05 contractions incl. operand packing)",
+                "kernel": "tcgen05 contractions (one-launch products, which cut their operands themselves, and packed ones with their packing)",
                 "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "peak_source": (f"of measured: bf16 burst {bf16} TFLOP/s (MEASURED_PEAKS.json) / {passes:.2f} "
                                 "MMA passes per algorithmic flop (mean over the step's products; TF32 passes count 2)"

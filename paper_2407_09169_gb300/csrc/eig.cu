@@ -18,12 +18,15 @@
 //      problems, and dc_order; single precision: eig_apply_rotations (one
 //      thread per row of the eigenvector matrix Z of the tridiagonal problem,
 //      over several blocks), which replays the rotation list on its row;
-//   3. eig_back_transform (four lanes per kept eigenvector): applies the
-//      Householder reflectors, U[:, r] = H_0 ... H_{n-3} Z[:, order[r]].
-// Every loop is bounded; a QL iteration stops after 60 sweeps per
-// eigenvalue (or when the rotation list is full), a secular root after 100
-// steps, and the two QL lanes wait on each other for at most about a second;
-// both report through the status word (bits 2 and 8).
+//   3. eig_back_transform_reg (FP64 up to n = 160: eight lanes per kept
+//      eigenvector, in registers) or eig_back_transform (four lanes, in shared
+//      memory): applies the Householder reflectors, U[:, r] = H_0 ... H_{n-3}
+//      Z[:, order[r]].
+// Every loop is bounded.  A QL iteration stops after 60 sweeps per eigenvalue
+// (or when the rotation list is full; status bit 2), and the two QL lanes wait
+// on each other for at most about a second (bit 8).  A secular root keeps the
+// value it has after 100 steps, inside its bracket, and reports nothing: the
+// vectors are formed from the recomputed z, orthogonal for any such roots.
 #include <algorithm>
 
 #include <cuda_runtime.h>
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(TRI_THREADS) eig_tridiag_ql(const EigProblem* 
     else if (c == i) W[L.A + x] = tauv[i];
   }
 
-  if (dc) {  // the tridiagonal (d, e) for eig_dc, which finds its eigenpairs
+  if (dc) {  // the tridiagonal (d, e) for the divide and conquer, which finds its eigenpairs
     for (int i = tid; i < n; i += TRI_THREADS) {
       W[L.dcv + i] = d[i];
       W[L.dcv + n + i] = e[i];
@@ -556,10 +559,12 @@ __global__ void __launch_bounds__(TRI_THREADS) eig_tridiag_ql(const EigProblem* 
 // z, eight columns of the product a block, a warp per leaf.  The reciprocals
 // are Newton steps on the hardware approximation (five instructions where the
 // division takes about ten).  The vectors alternate between Z and V from
-// level to level.  With it, the tridiagonalisation's look-ahead and the
-// four-lane back-transform: eigensolver class of the 40-site chi = 128 step
-// 8.1 -> 4.6 ms, truncation backward of 40 sites 11.5 -> 8.0 and of 20 sites
-// (n = 40) 3.5 -> 2.0, 20-site chi = 32 step 10.0 -> 8.1.
+// level to level.  With it, the tridiagonalisation's look-ahead and a
+// four-lane back-transform, the other kernels as they were then: eigensolver
+// class of the 40-site chi = 128 step 8.1 -> 4.6 ms, truncation backward of 40
+// sites 11.5 -> 8.0 and of 20 sites (n = 40) 3.5 -> 2.0, 20-site chi = 32 step
+// 10.0 -> 8.1.  Now, per stage of 25 problems of n = 136: leaves 160 us, roots
+// 440 (four levels), the other phases 210.
 constexpr int DC_LEAF = 12;
 constexpr int DC_SECULAR_ITERS = 100;
 constexpr int DC_THREADS = 128;

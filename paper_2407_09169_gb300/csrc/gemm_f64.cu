@@ -16,7 +16,7 @@
 // over all SMs in one launch, where 16 x 16 tiles gave 81 blocks and a K split
 // over the grid needs a reduction launch.  That one remains for products with
 // few outputs and a long K (the range product 272 x 136 x 16384).  Before and
-// after: step of 20 sites chi 32 15.3 -> 10.0 ms, of 30 sites chi 64 44.5 ->
+// after, the other kernels as they were then: step of 20 sites chi 32 15.3 -> 10.0 ms, of 30 sites chi 64 44.5 ->
 // 35.7; untruncated step of 10 sites 1.31 -> 0.40; truncation backward of 40
 // sites chi 128 13.6 -> 11.5; 40 sites chi 128 BF16X10 (its Grams) 57.1 -> 55.1.
 //

@@ -26,10 +26,12 @@
 // operand does not depend on the outer index, so ragged bonds fill their
 // tiles.  A long K (the range product) is split over CTAs, with the FP64
 // reduction of the packed GEMM.  Every wait is bounded.  Steps before and
-// after: 40 sites chi 128 BF16X10 51.2 -> 41.5 ms, 30 sites chi 64 FP32 15.4 ->
-// 12.9, an uneven grid chi 77 BF16X10 19.8 -> 16.0, 20 sites chi 32 BF16X10
-// 11.8 -> 5.4; half the launches (4068 -> 2067 at chi 128).  Distance to the
-// FP64 path after one step (30 sites, FP32, five seeds): 3.6e-6 -> 2.9e-6.
+// after, the other kernels as they were then: 40 sites chi 128 BF16X10 51.2 ->
+// 41.5 ms, 30 sites chi 64 FP32 15.4 -> 12.9, an uneven grid chi 77 BF16X10 19.8
+// -> 16.0, 20 sites chi 32 BF16X10 11.8 -> 5.4; half the launches (4068 -> 2067
+// at chi 128).  Distance to the FP64 path after one step of 30 sites, chi 64
+// (geometric mean over eight seeds, packed products -> these): FP32 3.0e-6 ->
+// 3.0e-6, BF16X10 3.4e-7 -> 2.4e-7.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -500,7 +502,8 @@ __global__ void __launch_bounds__(FT, 1) tc_fused_kernel(const FusedArgs g) {
   if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// K of one exact-slice product: its shifts and exponent fields have to fit.
+// K of one exact-slice product: its exponent fields have to fit the stage
+// buffers (asserted below); longer ones go to the packed GEMM.
 constexpr int fused_max_k(int mode) { return mode == TC_BF16X10 ? 448 : 352; }
 
 template <int MODE, int BN>
@@ -569,8 +572,16 @@ bool gemm_fused(cudaStream_t st, int mode, int M, int N, int K, int outer, int i
   // The tall side: the operand that may vary over the outer index gives the
   // rows (all outer entries flat), the other one the columns.
   const bool keep_ok = outer == 1 || B.so == 0, swap_ok = outer == 1 || A.so == 0;
-  // Wide column operands are converted once per row tile, and the rows once
-  // per column tile: beyond two or three tiles the packed GEMM is the better one.
+  // Wide column operands are converted once per row tile, and the rows once per
+  // column tile.  Alone and from a cold L2, row-major, K = 136 (this / packed, us):
+  // 17408 rows, BF16X6 136 columns 71 / 69, 208 102 / 89, 272 124 / 99, 400 178 /
+  // 135; TF32X3 30 / 36, 47 / 43, 56 / 54, 80 / 83; 272 rows, BF16X6 37 / 47, 42 /
+  // 35, 46 / 36, 43 / 36.  In whole steps the packed product's three to five
+  // launches weigh more: with the line at 144 columns the step takes 40 sites chi
+  // 128 38.5 -> 38.1 ms, uneven grid chi 77 14.3 -> 14.6, batch of 12 178 -> 180,
+  // a drawn one 13.3 -> 13.7, and the first step up to 70 ms more (the packed
+  // product's timed tile choices).  So the line takes 2 chi columns up to the
+  // bond 144 that the other limits (float QR in registers, field tables) have.
   constexpr int kMaxCols = 288;
   auto cost = [&](int m, int n) {  // elements converted
     const long long rt = ((long long)m * outer + BM - 1) / BM;

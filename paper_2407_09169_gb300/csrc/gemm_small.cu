@@ -18,7 +18,7 @@
 // One thread per column with all of M and K on it (the layout before) left a
 // 32 x 40 x 32 product with 32 batch entries on 40 warps at 78 us in FP64,
 // and the four pieces took four launches that re-read C.  Step before and
-// after: 20 sites chi 32 FP64 19.1 -> 15.3 ms, 30 sites chi 64 FP64 46.6 ->
+// after, the other kernels as they were then: 20 sites chi 32 FP64 19.1 -> 15.3 ms, 30 sites chi 64 FP64 46.6 ->
 // 44.5 and FP32 20.7 -> 19.5, 40 sites chi 128 BF16X10 59.7 -> 57.1.
 #include <algorithm>
 #include <cstdint>
